@@ -785,11 +785,19 @@ int build_context(cavmd_ctx *c, const cavmd_system *sys, const cavmd_sk_tables *
     std::vector<double> kpts;
     if (sys->lattice && kgrid_points(&c->opt) > 1) kpts = pbc_kpoints(c->opt.kgrid);
     const int nk = (int)(kpts.size() / 4);
+    bool water_order = true;   // every cell: 4, 1 and 1 orbitals in this order, eight electrons
     for (int n = 0; n < N; ++n) {
         int no = 0;
         for (int i = sys->cell_offset[n]; i < sys->cell_offset[n + 1]; ++i) no += sk->norb[sys->species[i]];
         if (!sys->lattice && (no != 6 || sys->cell_offset[n + 1] - sys->cell_offset[n] != 3)) c->generic = true;
         coff[n + 1] = coff[n] + (nk > 0 ? 4LL * nk : 1LL) * no * no;
+        if (no == 6 && sys->cell_offset[n + 1] - sys->cell_offset[n] == 3) {
+            const int32_t *sp = sys->species + sys->cell_offset[n];
+            const double nel = sk->zval[sp[0]] + sk->zval[sp[1]] + sk->zval[sp[2]];
+            if (sk->norb[sp[0]] != 4 || (int)((float)nel * 0.5f + 0.25f) != 4) water_order = false;
+        } else {
+            water_order = false;
+        }
     }
     c->n_cwarm = coff[N];
     AL(c->d_qpop, NA); AL(c->d_qprev, NA); AL(c->d_C, (size_t)coff[N]); AL(c->d_E, N); AL(c->d_Mc, N);
@@ -1025,6 +1033,7 @@ int build_context(cavmd_ctx *c, const cavmd_system *sys, const cavmd_sk_tables *
     d.max_iter = c->opt.scc_max_iter;
     d.hist = c->opt.scc_history;
     d.have_warm = 0;
+    d.warm_water = water_order && !c->periodic;
     d.max_sweeps = c->opt.jacobi_max_sweeps;
     d.write_b = c->opt.charge_model == CAVMD_CHARGE_MULLIKEN;
     d.n_disp = 0;
