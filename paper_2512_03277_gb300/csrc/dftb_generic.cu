@@ -33,6 +33,13 @@ constexpr double G_JACOBI_TOL = 1e-15;
 constexpr double G_MIN_GAP = 1e-3;
 constexpr double G_EIG_TOL = 1e-10;
 constexpr float G_KMAX_PERT = 1e-4f;
+constexpr int GW_FP32_ITERS = 5;       // warm path: bound on the FP32 Newton steps,
+constexpr float GW_FP32_KTOL = 3e-5f;  // the rotation below which the next step would be FP32 rounding
+constexpr float GW_ROT_MAX = 0.3f;     // the largest rotation taken (beyond: the general path)
+constexpr int GW_EVALS = 8;            // and bound on the FP64 evaluations
+constexpr float GW_ORTH_MAX = 1e-4f;   // overlap defect that the second-order correction takes
+constexpr float GW_GAP = 2e-3f;        // HOMO-LUMO gap (Hartree) the warm path needs, above G_MIN_GAP
+constexpr int GW_CG_ITERS = 40;        // bound on the conjugate-gradient steps of a Newton step
 constexpr int BT = 128;                // threads per block
 constexpr int TB = 128;                // threads per large cell
 constexpr int TS = 64;                 // threads per small cell (two per block)
@@ -40,9 +47,13 @@ constexpr int TS = 64;                 // threads per small cell (two per block)
 // Shared-memory layout of one cell (byte offsets) for cells of at most nmax orbitals, amax atoms.
 struct GLayout {
     int nmax, amax, pmax;
-    unsigned SH, C, A, Y, Kc, pos, gam, zv, q, qout, qst, shift, shl, hq, hf, red, diag, cs, invd, th, ints,
+    unsigned SH, C, A, Y, Kc, XB, pos, gam, zv, q, qout, qst, shift, shl, hq, hf, red, diag, cs, invd, th, ints,
         total;
 };
+
+// Doubles of the warm path's n x n_occ buffer (three quarters of an n x (n + 1) matrix: water
+// clusters need two thirds; cells with more occupied orbitals take the general path).
+__host__ __device__ inline int g_xb(int nmax) { return (3 * nmax + 3) / 4 * (nmax + 1); }
 
 __host__ __device__ inline GLayout g_layout(int nmax, int amax) {
     GLayout L;
@@ -58,6 +69,7 @@ __host__ __device__ inline GLayout g_layout(int nmax, int amax) {
     L.A = o; o += mat;
     L.Y = o; o += ymat;
     L.Kc = o; o += (unsigned)((nmax / 2) * ((nmax + 1) / 2) + 8) * 8;   // n_occ x n_virt <= n^2 / 4
+    L.XB = o; o += (unsigned)g_xb(nmax) * 8;
     L.pos = o; o += amax * 3 * 8;
     L.gam = o; o += amax * amax * 8;
     L.zv = o; o += amax * 8;
@@ -177,6 +189,503 @@ __device__ __forceinline__ void flat(int tid, int n_out, int nk, int xs, int zs,
         for (int r = 0; r < R; ++r)
             if (e0 + r * T < n_out) epi(e0 + r * T, acc[r]);
     }
+}
+
+// FP32 product in register tiles: for i < m, c < w, epi(i, c, sum_{k < K} X[i xi + k xk] Z[k zk + c zc]),
+// TM x TN entries per thread (clamped at the edges, the surplus dropped).
+template <int T, int TM, int TN, typename EPI>
+__device__ __forceinline__ void ftile(int tid, int m, int w, int K, const float *X, int xi, int xk, const float *Z,
+                                      int zk, int zc, EPI epi) {
+    const int ni = (m + TM - 1) / TM, nc = (w + TN - 1) / TN;
+    for (int t = tid; t < ni * nc; t += T) {
+        const int tc = t / ni, i0 = (t - tc * ni) * TM, c0 = tc * TN;
+        const float *xp[TM], *zp[TN];
+        float acc[TM][TN];
+#pragma unroll
+        for (int r = 0; r < TM; ++r) xp[r] = X + min(i0 + r, m - 1) * xi;
+#pragma unroll
+        for (int c = 0; c < TN; ++c) zp[c] = Z + min(c0 + c, w - 1) * zc;
+#pragma unroll
+        for (int r = 0; r < TM; ++r)
+#pragma unroll
+            for (int c = 0; c < TN; ++c) acc[r][c] = 0.0f;
+#pragma unroll 2
+        for (int k = 0; k < K; ++k) {
+            float x[TM], z[TN];
+#pragma unroll
+            for (int r = 0; r < TM; ++r) x[r] = xp[r][k * xk];
+#pragma unroll
+            for (int c = 0; c < TN; ++c) z[c] = zp[c][k * zk];
+#pragma unroll
+            for (int r = 0; r < TM; ++r)
+#pragma unroll
+                for (int c = 0; c < TN; ++c) acc[r][c] = fmaf(x[r], z[c], acc[r][c]);
+        }
+#pragma unroll
+        for (int r = 0; r < TM; ++r)
+#pragma unroll
+            for (int c = 0; c < TN; ++c)
+                if (i0 + r < m && c0 + c < w) epi(i0 + r, c0 + c, acc[r][c]);
+    }
+}
+
+// Column c and row i >= c of entry e of the packed lower triangle (column by column) of an m x m matrix.
+__device__ __forceinline__ void g_lower(int e, int m, int &i, int &c) {
+    const float b = 2.0f * (float)m + 1.0f;
+    c = (int)((b - sqrtf(fmaxf(b * b - 8.0f * (float)e, 0.0f))) * 0.5f);
+    c = max(0, min(c, m - 1));
+    while (c > 0 && c * m - c * (c - 1) / 2 > e) --c;
+    while (c + 1 < m && (c + 1) * m - (c + 1) * c / 2 <= e) ++c;
+    i = c + (e - (c * m - c * (c - 1) / 2));
+}
+
+// What the warm path works on (shared memory of one cell, see GLayout).
+struct GWarm {
+    int n, nocc, nat, AM;
+    double *SH, *A, *XB, *Kc, *gam, *zv, *q, *shift, *red;
+    float *u, *dq, *ea, *eo, *scr;   // [n], [nat], [nat], [n], [8]: FP32 charges, shifts, reduction scratch
+    const int *orb_atom, *atom_off;
+};
+
+// Warm-started cell: the method of k_water_warm (dftb_kernel.cu) for matrices of any size.
+//
+// The general path below spends 10.8 FP64 iterations of about 3.2 n^3 multiply-adds on a cell, and
+// FP64 multiply-adds are this kernel's bound. Here the previous basis (occupied columns first) is
+// made orthonormal under the new overlap and moved by Newton steps of the orbital rotation in FP32
+// (64 times the FP64 rate), each step solved by conjugate gradients on the orbital Hessian
+//   K -> A_vv K - K A_oo + C_v^T dH(K) C_o,  dH = S o (e_A + e_B) / 2, e = gamma dq(K),
+// preconditioned by the diagonal differences (3 to 7 iterations). Two steps reach FP32 rounding. Then
+// in FP64: the orthonormal correction C (1 - E/2 + 3/8 E^2); evaluations of q(C), H(q), H C_o and the
+// residual A_vo, each followed by the rotation C (1 + K + K^2/2) with K from the FP32 Hessian of this
+// basis. Converged when every |A_vo| < G_EIG_TOL and the populations that A_vo implies to first
+// order, q_out - q, are below scc_tol: two or three evaluations, about 9 n^3 FP64 multiply-adds with
+// the correction. Nothing of the FP32 part but the starting basis and the approximate Hessian enters
+// the result. Returns false, with SH untouched, for a cell that leaves the path's range (a large
+// rotation or overlap change, a Hessian or gap that is not safely positive, no convergence): the
+// general path takes it. On success: C (FP64, occupied columns first), q, shift, XB = H C_o.
+// Measured (GB300, one launch of 16,384 clusters (H2O)_1..8): 84 -> 24 ms, mean evaluations 2.0 against
+// 10.8 iterations; 301 clusters 4.9 -> 1.1 ms. Bound: the FP64 pipe (55 % busy with eight warps per SM).
+template <int T, int R>
+__device__ bool g_warm(const DftbArgs &a, const GWarm &v, double *&C, double *&Y, const double *cw, const Grp<T> &g,
+                       int &evals) {
+    const int j = g.tid;
+    const int n = v.n, no = v.nocc, nv = n - no, nat = v.nat, LD = n + 1, LF = n + 1, nn = n * n, nvo = nv * no;
+    double *SH = v.SH, *A = v.A, *XB = v.XB;
+    // FP32 matrices in the halves of the FP64 buffers, row-major with stride LF
+    float *F0 = (float *)Y, *F1 = F0 + n * LF, *F2 = (float *)A, *F3 = F2 + n * LF;
+    float *F4 = (float *)C, *F5 = F4 + n * LF;
+    float *x = (float *)v.Kc, *r = x + nvo;   // K and the residual, [virtual][occupied]
+    auto s_at = [&](int i, int k) -> double {
+        const double lo = SH[k * LD + i], up = SH[i * LD + k];
+        return i == k ? 1.0 : (i > k ? lo : up);
+    };
+    auto h0_at = [&](int i, int k) -> double {
+        const double lo = SH[k * LD + i], up = SH[i * LD + k];
+        return i <= k ? lo : up;
+    };
+    auto all = [&](bool p) { return g.all(p); };
+    auto sum = [&](float s) -> float {   // over the group, in a fixed order
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(CAVMD_FULL_MASK, s, o);
+        g.sync();
+        if ((j & 31) == 0) v.scr[j >> 5] = s;
+        g.sync();
+        float t = v.scr[0];
+#pragma unroll
+        for (int w = 1; w < T / 32; ++w) t += v.scr[w];
+        return t;
+    };
+    auto s32 = [&]() {
+        for (int e = j; e < nn; e += T) {
+            const int c = e / n, i = e - c * n;
+            F2[c * LF + i] = d2f_steer(s_at(i, c));
+        }
+        g.sync();
+    };
+    // F1 = S F0 (S32 in F2)
+    auto sc32 = [&]() {
+        ftile<T, 6, 3>(j, n, n, n, F2, 1, LF, F0, LF, 1, [&](int i, int c, float t) { F1[i * LF + c] = t; });
+        g.sync();
+    };
+    // A32 = F0^T H F0 into F2, H with the orbital half shifts eo (F3 holds H F0 on the way)
+    auto a32 = [&]() {
+        for (int e = j; e < nn; e += T) {
+            const int c = e / n, i = e - c * n;
+            F2[c * LF + i] = fmaf(d2f_steer(s_at(i, c)), v.eo[i] + v.eo[c], d2f_steer(h0_at(i, c)));
+        }
+        g.sync();
+        ftile<T, 6, 3>(j, n, n, n, F2, 1, LF, F0, LF, 1, [&](int i, int c, float t) { F3[i * LF + c] = t; });
+        g.sync();
+        ftile<T, 6, 3>(j, n, n, n, F0, 1, LF, F3, LF, 1, [&](int i, int c, float t) { F2[i * LF + c] = t; });
+        g.sync();
+    };
+    // populations moved by K = kv to first order, per atom into dq; uses F0 = C, F1 = S C and F3's tail
+    auto charges = [&](const float *kv) {
+        float *part = F3 + 2 * nvo;
+        const int ni = (n + 5) / 6, nc = (no + 1) / 2;
+        for (int t = j; t < ni * nc; t += T) {
+            const int tc = t / ni, i0 = (t - tc * ni) * 6, c0 = 2 * tc, c1 = min(2 * tc + 1, no - 1);
+            float ax[6][2], as[6][2];
+            const float *cp[6], *sp[6];
+#pragma unroll
+            for (int q = 0; q < 6; ++q) {
+                cp[q] = F0 + min(i0 + q, n - 1) * LF;
+                sp[q] = F1 + min(i0 + q, n - 1) * LF;
+                ax[q][0] = ax[q][1] = as[q][0] = as[q][1] = 0.0f;
+            }
+            for (int k = 0; k < nv; ++k) {
+                const float k0 = kv[k * no + c0], k1 = kv[k * no + c1];
+#pragma unroll
+                for (int q = 0; q < 6; ++q) {
+                    const float cv = cp[q][no + k], sv = sp[q][no + k];
+                    ax[q][0] = fmaf(cv, k0, ax[q][0]);
+                    ax[q][1] = fmaf(cv, k1, ax[q][1]);
+                    as[q][0] = fmaf(sv, k0, as[q][0]);
+                    as[q][1] = fmaf(sv, k1, as[q][1]);
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < 6; ++q) {
+                if (i0 + q >= n) continue;
+                float s = fmaf(ax[q][0], sp[q][c0], cp[q][c0] * as[q][0]);
+                if (c0 + 1 < no) s += fmaf(ax[q][1], sp[q][c1], cp[q][c1] * as[q][1]);
+                part[tc * n + i0 + q] = s;
+            }
+        }
+        g.sync();
+        if (j < n) {
+            float s = 0.0f;
+            for (int t = 0; t < nc; ++t) s += part[t * n + j];
+            v.u[j] = 2.0f * s;
+        }
+        g.sync();
+        if (j < nat) {
+            float s = 0.0f;
+            for (int o = v.atom_off[j]; o < v.atom_off[j + 1]; ++o) s += v.u[o];
+            v.dq[j] = s;
+        }
+        g.sync();
+    };
+    // half shifts of the orbitals from the atoms' charges dq
+    auto half_shifts = [&]() {
+        if (j < nat) {
+            float s = 0.0f;
+            for (int k = 0; k < nat; ++k) s = fmaf(d2f_steer(v.gam[j * v.AM + k]), v.dq[k], s);
+            v.ea[j] = 0.5f * s;
+        }
+        g.sync();
+        if (j < n) v.eo[j] = v.ea[v.orb_atom[j]];
+        g.sync();
+    };
+    auto diag_of = [&](int e) -> float {
+        const int vi = e / no, o = e - vi * no;
+        return F2[(no + vi) * LF + no + vi] - F2[o * LF + o];
+    };
+    // K (in x) from the residual r (destroyed): Hessian K = r to a relative residual rel, by
+    // preconditioned conjugate gradients. False when the Hessian is not positive along the way.
+    auto newton = [&](float rel) -> bool {
+        float *p = F3, *hp = F3 + nvo;
+        float rz = 0.0f;
+        for (int e = j; e < nvo; e += T) {
+            const float z = r[e] / diag_of(e);
+            x[e] = 0.0f;
+            p[e] = z;
+            rz = fmaf(r[e], z, rz);
+        }
+        rz = sum(rz);
+        const float stop = rel * rel * rz;
+        if (!(rz < 1e30f) || !(rz >= 0.0f)) return false;
+        for (int it = 0; it < GW_CG_ITERS && rz > stop; ++it) {
+            charges(p);
+            half_shifts();
+            ftile<T, 2, 2>(j, nv, no, nv, F2 + no * LF + no, LF, 1, p, no, 1,
+                           [&](int i, int c, float t) { hp[i * no + c] = t; });
+            ftile<T, 2, 2>(j, nv, no, no, p, no, 1, F2, LF, 1, [&](int i, int c, float t) { hp[i * no + c] -= t; });
+            {   // C_v^T (e S C_o) + (S C_v)^T (e C_o): the same tiles, so each thread adds to its own entries
+                const int ni = (nv + 1) / 2, nc = (no + 1) / 2;
+                for (int t = j; t < ni * nc; t += T) {
+                    const int tc = t / ni, i0 = 2 * (t - tc * ni), i1 = min(i0 + 1, nv - 1), c0 = 2 * tc, c1 = min(c0 + 1, no - 1);
+                    float a00 = 0.f, a01 = 0.f, a10 = 0.f, a11 = 0.f;
+                    for (int m = 0; m < n; ++m) {
+                        const float *cr = F0 + m * LF, *sr = F1 + m * LF;
+                        const float e = v.eo[m];
+                        const float s0 = e * sr[c0], s1 = e * sr[c1], q0 = e * cr[c0], q1 = e * cr[c1];
+                        const float v0 = cr[no + i0], v1 = cr[no + i1], w0 = sr[no + i0], w1 = sr[no + i1];
+                        a00 = fmaf(v0, s0, fmaf(w0, q0, a00));
+                        a01 = fmaf(v0, s1, fmaf(w0, q1, a01));
+                        a10 = fmaf(v1, s0, fmaf(w1, q0, a10));
+                        a11 = fmaf(v1, s1, fmaf(w1, q1, a11));
+                    }
+                    hp[i0 * no + c0] += a00;
+                    if (c0 + 1 < no) hp[i0 * no + c1] += a01;
+                    if (i0 + 1 < nv) hp[i1 * no + c0] += a10;
+                    if (i0 + 1 < nv && c0 + 1 < no) hp[i1 * no + c1] += a11;
+                }
+            }
+            g.sync();
+            float ph = 0.0f;
+            for (int e = j; e < nvo; e += T) ph = fmaf(p[e], hp[e], ph);
+            ph = sum(ph);
+            if (!(ph > 0.0f)) return false;
+            const float al = rz / ph;
+            float rn = 0.0f;
+            for (int e = j; e < nvo; e += T) {
+                x[e] = fmaf(al, p[e], x[e]);
+                const float q = fmaf(-al, hp[e], r[e]);
+                r[e] = q;
+                rn = fmaf(q, q / diag_of(e), rn);
+            }
+            rn = sum(rn);
+            const float be = rn / rz;
+            rz = rn;
+            for (int e = j; e < nvo; e += T) p[e] = fmaf(be, p[e], r[e] / diag_of(e));
+            g.sync();
+        }
+        g.sync();
+        return true;
+    };
+    // second-order parts of the rotation: G[i][o] = 1/2 sum_v C[i][v] K_vo, G[i][no + v] = -1/2 sum_o C[i][o] K_vo
+    auto second = [&](float *G, bool with_c) {
+        ftile<T, 6, 2>(j, n, no, nv, F0 + no, LF, 1, x, no, 1, [&](int i, int c, float t) {
+            G[i * LF + c] = fmaf(0.5f, t, with_c ? F0[i * LF + c] : 0.0f);
+        });
+        ftile<T, 3, 2>(j, n, nv, no, F0, LF, 1, x, 1, no, [&](int i, int c, float t) {
+            G[i * LF + no + c] = fmaf(-0.5f, t, with_c ? F0[i * LF + no + c] : 0.0f);
+        });
+        g.sync();
+    };
+
+    // ---------------------------------------------------------------- FP32 start
+    for (int e = j; e < nn; e += T) {
+        const int c = e / n, i = e - c * n;
+        F0[i * LF + c] = d2f_steer(cw[e]);
+    }
+    s32();
+    for (int pass = 0; pass < 2; ++pass) {   // E is a few 1e-2 after one step: below 1e-6 after two passes
+        sc32();
+        float big = 0.0f;
+        ftile<T, 6, 3>(j, n, n, n, F0, 1, LF, F1, LF, 1, [&](int i, int c, float t) {
+            const float e = t - (i == c ? 1.0f : 0.0f);
+            big = fmaxf(big, fabsf(e));
+            if (pass == 0) F3[i * LF + c] = e;
+            else F4[i * LF + c] = fmaf(-0.5f, e, i == c ? 1.0f : 0.0f);
+        });
+        if (!all(big < 0.2f)) return false;   // NaN included
+        if (pass == 0) {
+            g.sync();
+            ftile<T, 6, 3>(j, n, n, n, F3, 1, LF, F3, LF, 1, [&](int i, int c, float t) {
+                F4[i * LF + c] = fmaf(0.375f, t, fmaf(-0.5f, F3[i * LF + c], i == c ? 1.0f : 0.0f));
+            });
+        }
+        g.sync();
+        ftile<T, 6, 3>(j, n, n, n, F0, LF, 1, F4, LF, 1, [&](int i, int c, float t) { F5[i * LF + c] = t; });
+        g.sync();
+        for (int e = j; e < nn; e += T) {
+            const int i = e / n, c = e - i * n;
+            F0[i * LF + c] = F5[i * LF + c];
+        }
+        g.sync();
+    }
+    bool done = false;
+    for (int it = 0; it < GW_FP32_ITERS && !done; ++it) {
+        if (it > 0) s32();
+        sc32();
+        if (j < n) {
+            float s = 0.0f;
+            for (int o = 0; o < no; ++o) s = fmaf(F0[j * LF + o], F1[j * LF + o], s);
+            v.u[j] = 2.0f * s;
+        }
+        g.sync();
+        if (j < nat) {
+            float s = -d2f_steer(v.zv[j]);
+            for (int o = v.atom_off[j]; o < v.atom_off[j + 1]; ++o) s += v.u[o];
+            v.dq[j] = s;
+        }
+        g.sync();
+        half_shifts();
+        a32();
+        for (int e = j; e < nvo; e += T) {
+            const int vi = e / no, o = e - vi * no;
+            r[e] = -0.5f * (F2[(no + vi) * LF + o] + F2[o * LF + no + vi]);
+        }
+        g.sync();
+        if (!newton(it < 2 ? 3e-3f : 1e-2f)) return false;
+        float kmax = 0.0f;
+        for (int e = j; e < nvo; e += T) kmax = fmaxf(kmax, fabsf(x[e]));
+        if (!all(kmax < GW_ROT_MAX)) return false;
+        done = all(kmax < GW_FP32_KTOL);
+        second(F4, true);
+        ftile<T, 6, 2>(j, n, no, nv, F4 + no, LF, 1, x, no, 1, [&](int i, int c, float t) { F0[i * LF + c] += t; });
+        ftile<T, 3, 2>(j, n, nv, no, F4, LF, 1, x, 1, no, [&](int i, int c, float t) { F0[i * LF + no + c] -= t; });
+        g.sync();
+    }
+    if (!done) return false;
+
+    // ---------------------------------------------------------------- FP64: orthonormal basis
+    for (int e = j; e < nn; e += T) {
+        const int c = e / n, i = e - c * n;
+        C[c * LD + i] = f2d_steer(F0[i * LF + c]);
+        A[c * LD + i] = s_at(i, c);
+    }
+    g.sync();
+    flat<T, R>(j, nn, n, LD, 1, [&](int e) { return A + (e % n); }, [&](int e) { return C + (e / n) * LD; },
+               [&](int e, double t) { Y[(e / n) * LD + e % n] = t; });
+    g.sync();
+    {   // E = C^T S C - 1 into A, and in FP32 into XB
+        float *E32 = (float *)XB;
+        float big = 0.0f;
+        flat<T, R>(j, n * (n + 1) / 2, n, 1, 1,
+                   [&](int e) { int i, c; g_lower(e, n, i, c); return C + i * LD; },
+                   [&](int e) { int i, c; g_lower(e, n, i, c); return Y + c * LD; }, [&](int e, double t) {
+                       int i, c;
+                       g_lower(e, n, i, c);
+                       if (i == c) t -= 1.0;
+                       A[c * LD + i] = t;
+                       A[i * LD + c] = t;
+                       const float f = d2f_steer(t);
+                       E32[c * LF + i] = f;
+                       E32[i * LF + c] = f;
+                       big = fmaxf(big, fabsf(f));
+                   });
+        if (!all(big < GW_ORTH_MAX)) return false;
+        g.sync();
+        // 1 - E/2 + 3/8 E^2: E^2 is below 1e-8, so FP32 carries it beyond FP64 rounding
+        ftile<T, 6, 3>(j, n, n, n, E32, 1, LF, E32, LF, 1, [&](int i, int c, float t) {
+            A[c * LD + i] = fma(-0.5, A[c * LD + i], (i == c ? 1.0 : 0.0) + f2d_steer(0.375f * t));
+        });
+        g.sync();
+        flat<T, R>(j, nn, n, LD, 1, [&](int e) { return C + (e % n); }, [&](int e) { return A + (e / n) * LD; },
+                   [&](int e, double t) { Y[(e / n) * LD + e % n] = t; });
+        g.sync();
+        double *t = C;
+        C = Y;
+        Y = t;
+        F0 = (float *)Y;
+        F1 = F0 + n * LF;
+    }
+
+    // ---------------------------------------------------------------- FP64 evaluations
+    const int most = min(a.max_iter, GW_EVALS);
+    for (int it = 1; it <= most; ++it) {
+        for (int e = j; e < nn; e += T) {
+            const int c = e / n, i = e - c * n;
+            A[c * LD + i] = s_at(i, c);
+        }
+        g.sync();
+        flat<T, R>(j, n * no, n, LD, 1, [&](int e) { return A + (e % n); }, [&](int e) { return C + (e / n) * LD; },
+                   [&](int e, double t) { XB[(e / n) * LD + e % n] = t; });
+        g.sync();
+        if (j < n) {
+            double t = 0.0;
+            for (int o = 0; o < no; ++o) t = fma(C[o * LD + j], XB[o * LD + j], t);
+            v.red[j] = 2.0 * t;
+        }
+        g.sync();
+        if (j < nat) {
+            double t = 0.0;
+            for (int o = v.atom_off[j]; o < v.atom_off[j + 1]; ++o) t += v.red[o];
+            v.q[j] = t;
+        }
+        g.sync();
+        if (j < nat) {
+            double t = 0.0;
+            for (int k = 0; k < nat; ++k) t = fma(v.gam[j * v.AM + k], v.q[k] - v.zv[k], t);
+            v.shift[j] = t;
+        }
+        g.sync();
+        if (j < n) v.eo[j] = 0.5f * d2f_steer(v.shift[v.orb_atom[j]]);
+        for (int e = j; e < nn; e += T) {
+            const int c = e / n, i = e - c * n;
+            A[c * LD + i] = fma(0.5 * s_at(i, c), v.shift[v.orb_atom[i]] + v.shift[v.orb_atom[c]], h0_at(i, c));
+        }
+        g.sync();
+        flat<T, R>(j, n * no, n, LD, 1, [&](int e) { return A + (e % n); }, [&](int e) { return C + (e / n) * LD; },
+                   [&](int e, double t) { XB[(e / n) * LD + e % n] = t; });
+        g.sync();
+        bool small = true, finite = true;
+        flat<T, R>(j, nvo, n, 1, 1, [&](int e) { return C + (no + e / no) * LD; },
+                   [&](int e) { return XB + (e % no) * LD; }, [&](int e, double t) {
+                       if (!abs_lt(t, G_EIG_TOL)) small = false;
+                       if (!abs_lt(t, 1.0)) finite = false;
+                       r[e] = -d2f_steer(t);
+                   });
+        small = all(small);
+        if (!all(finite)) return false;
+        // the FP32 Hessian of this basis (over A and Y)
+        for (int e = j; e < nn; e += T) {
+            const int c = e / n, i = e - c * n;
+            F0[i * LF + c] = d2f_steer(C[c * LD + i]);
+        }
+        s32();
+        sc32();
+        a32();
+        if (small) {   // q_out - q to first order: K0 = r / (A_vv - A_oo)
+            for (int e = j; e < nvo; e += T) x[e] = r[e] / diag_of(e);
+            g.sync();
+            charges(x);
+            bool conv = true;
+            if (j < nat) conv = fabsf(v.dq[j]) < (float)a.scc_tol;
+            if (all(conv)) {
+                // aufbau and gap: tau - A_oo and A_vv - tau - GW_GAP positive definite (Cholesky pivots)
+                float hi = -1e30f, lo = 1e30f;
+                for (int o = 0; o < no; ++o) hi = fmaxf(hi, F2[o * LF + o]);
+                for (int k = no; k < n; ++k) lo = fminf(lo, F2[k * LF + k]);
+                const float tau = 0.5f * (hi + lo);
+                g.sync();
+                for (int e = j; e < nn; e += T) {
+                    const int i = e / n, c = e - i * n;
+                    if (i < no && c < no) F2[i * LF + c] = (i == c ? tau : 0.0f) - F2[i * LF + c];
+                    else if (i == c) F2[i * LF + c] -= tau + GW_GAP;
+                }
+                g.sync();
+                bool pd = true;
+                for (int k = 0; k < n; ++k) {   // both blocks in turn; entries between them are not touched
+                    const float d = F2[k * LF + k];
+                    pd = pd && d > 0.0f;
+                    const int end = k < no ? no : n;
+                    const float id = 1.0f / d;
+                    for (int i = k + 1 + j; i < end; i += T) {
+                        const float f = F2[i * LF + k] * id;
+                        for (int c = k + 1; c <= i; ++c) F2[i * LF + c] = fmaf(-f, F2[c * LF + k], F2[i * LF + c]);
+                    }
+                    g.sync();
+                }
+                if (!all(pd)) return false;
+                evals = it;
+                return true;
+            }
+        }
+        if (it == most || !newton(1e-6f)) return false;
+        float kmax = 0.0f;
+        for (int e = j; e < nvo; e += T) kmax = fmaxf(kmax, fabsf(x[e]));
+        if (!all(kmax < 1e-2f)) return false;
+        // C (1 + K + K^2/2), as C_o + (C_v - (C_o K^T)/2) K and C_v - (C_o + (C_v K)/2) K^T
+        second(F1, false);
+        double Kd[8];   // this thread's entries of K: n_virt n_occ <= n^2 / 4, 1024 on 128 threads at n = 64, 256 on 64 at n = 32
+#pragma unroll
+        for (int t = 0; t < 8; ++t) {
+            const int e = j + t * T;
+            Kd[t] = e < nvo ? f2d_steer(x[e]) : 0.0;
+        }
+        for (int e = j; e < nn; e += T) {
+            const int c = e / n, i = e - c * n;
+            A[c * LD + i] = C[c * LD + i] + f2d_steer(F1[i * LF + c]);
+        }
+        g.sync();
+        double *K = v.Kc;
+#pragma unroll
+        for (int t = 0; t < 8; ++t) {
+            const int e = j + t * T;
+            if (e < nvo) K[e] = Kd[t];
+        }
+        g.sync();
+        flat<T, R>(j, n * no, nv, LD, no, [&](int e) { return A + no * LD + e % n; }, [&](int e) { return K + e / n; },
+                   [&](int e, double t) { C[(e / n) * LD + e % n] += t; });
+        flat<T, R>(j, n * nv, no, LD, 1, [&](int e) { return A + e % n; }, [&](int e) { return K + (e / n) * no; },
+                   [&](int e, double t) { C[(no + e / n) * LD + e % n] -= t; });
+        g.sync();
+    }
+    return false;
 }
 
 // One cell (main evaluation, kd < 0) or one displaced copy of it (kd = displacement index),
@@ -315,9 +824,27 @@ __device__ void g_molecule(const DevSK &sk, const DftbArgs &a, const GLayout &L,
         }
     }
 
-    // ---------------------------------------------------------------- warm-started S-orthonormal basis
     const long long coff = a.Cwarm_off ? a.Cwarm_off[cell] : (long long)cell * 36;
     const double *cw = a.Cwarm + coff;
+    // ---------------------------------------------------------------- warm path
+    bool warm = false;
+    if (a.have_warm && nocc > 0 && nv > 0 && nocc * LD <= g_xb(L.nmax)) {
+        GWarm wv;
+        wv.n = n; wv.nocc = nocc; wv.nat = nat; wv.AM = AM;
+        wv.SH = SH; wv.A = A; wv.XB = (double *)(sm + L.XB); wv.Kc = Kc; wv.gam = gam; wv.zv = zv; wv.q = q;
+        wv.shift = shift; wv.red = red;
+        wv.u = (float *)diag; wv.dq = (float *)qout; wv.ea = (float *)shl; wv.eo = (float *)invd; wv.scr = (float *)th;
+        wv.orb_atom = orb_atom; wv.atom_off = atom_off;
+        g.sync();
+        int evals = 0;
+        warm = g_warm<T, R>(a, wv, C, Y, cw, g, evals);
+        g.sync();
+        if (warm && j == 0) fl[2] = evals;
+        if (warm && j < nat) qst[j] = a.qpop[a0 + j];
+        g.sync();
+    }
+    if (!warm) {
+    // ---------------------------------------------------------------- warm-started S-orthonormal basis
     for (int e = j; e < nn; e += T) {   // coalesced copy of the previous eigenvectors
         const int c = e / n, i = e - c * n;
         C[c * LD + i] = a.have_warm ? cw[e] : (i == c ? 1.0 : 0.0);
@@ -627,6 +1154,7 @@ __device__ void g_molecule(const DevSK &sk, const DftbArgs &a, const GLayout &L,
         fl[2] = a.max_iter;
     }
     g.sync();
+    }   // general path
 
     if (disp) {   // displaced copy: only the dipole of the converged charges
         if (j == 0) {
@@ -643,11 +1171,63 @@ __device__ void g_molecule(const DevSK &sk, const DftbArgs &a, const GLayout &L,
     }
 
     // ---------------------------------------------------------------- energy, forces, dipole
-    {   // eigenvectors for the next warm start
+    const double *P = C, *W = SH;
+    if (warm) {
+        // W = 2 C_o A_oo C_o^T and P = 2 C_o C_o^T with A_oo = C_o^T (H C_o) of the last evaluation: A <- A_oo;
+        // Y <- t = 2 A_oo C_o^T; A <- P and SH <- W, the entries above the diagonal (all that the pair
+        // gradients read). Band energy: Tr P H0 = 2 Tr A_oo - sum_A q_A eps_A.
+        const double *XB = (const double *)(sm + L.XB);
         double *cwo = a.Cwarm + coff;
         for (int e = j; e < nn; e += T) {
             const int c = e / n;
             cwo[e] = C[c * LD + (e - c * n)];
+        }
+        flat<T, R>(j, nocc * (nocc + 1) / 2, n, 1, 1,
+                   [&](int e) { int i, c; g_lower(e, nocc, i, c); return C + i * LD; },
+                   [&](int e) { int i, c; g_lower(e, nocc, i, c); return XB + c * LD; }, [&](int e, double v) {
+                       int i, c;
+                       g_lower(e, nocc, i, c);
+                       A[c * LD + i] = v;
+                       A[i * LD + c] = v;
+                   });
+        g.sync();
+        if (j == 0) {
+            double eb = 0.0;
+            for (int o = 0; o < nocc; ++o) eb += A[o * LD + o];
+            eb *= 2.0;
+            for (int at = 0; at < nat; ++at) eb = fma(-q[at], shift[at], eb);
+            red[0] = eb;
+        }
+        if (j > 0 && j < n) red[j] = 0.0;
+        // t(o, i) = 2 sum_p A_oo(o, p) C(i, p) into Y[i * LD + o]
+        flat<T, R>(j, nocc * n, nocc, LD, LD, [&](int e) { return A + (e % nocc); }, [&](int e) { return C + (e / nocc); },
+                   [&](int e, double v) { Y[(e / nocc) * LD + e % nocc] = 2.0 * v; });
+        g.sync();
+        if (n > 1) {   // entries (row c, column i), c < i: the strict lower triangle (i, c) transposed
+            flat<T, R>(j, n * (n - 1) / 2, nocc, LD, LD,
+                       [&](int e) { int i, c; g_lower(e, n - 1, i, c); return C + i + 1; },
+                       [&](int e) { int i, c; g_lower(e, n - 1, i, c); return C + c; }, [&](int e, double v) {
+                           int i, c;
+                           g_lower(e, n - 1, i, c);
+                           A[(i + 1) * LD + c] = 2.0 * v;
+                       });
+            flat<T, R>(j, n * (n - 1) / 2, nocc, 1, LD,
+                       [&](int e) { int i, c; g_lower(e, n - 1, i, c); return Y + (i + 1) * LD; },
+                       [&](int e) { int i, c; g_lower(e, n - 1, i, c); return C + c; }, [&](int e, double v) {
+                           int i, c;
+                           g_lower(e, n - 1, i, c);
+                           SH[(i + 1) * LD + c] = v;
+                       });
+        }
+        if (j < nat) shl[j] = shift[j];
+        g.sync();
+        P = A;
+    } else {
+    {   // eigenvectors for the next warm start
+        double *cwo = a.Cwarm + coff;
+        for (int e = j; e < nn; e += T) {   // occupied columns first, as the warm path reads them
+            const int c = e / n, src = c < nocc ? occ_list[c] : virt_list[c - nocc];
+            cwo[e] = C[src * LD + (e - c * n)];
         }
     }
     if (j < nat) {
@@ -699,7 +1279,8 @@ __device__ void g_molecule(const DevSK &sk, const DftbArgs &a, const GLayout &L,
     flat<T, R>(j, nn, nocc, LD, 1, [&](int e) { return A + (e % n); }, [&](int e) { return Y + (e / n) * LD; },
                [&](int e, double v) { SH[(e / n) * LD + e % n] = v; });
     g.sync();
-    const double *P = C, *W = SH;
+    P = C;
+    }
     double *gp = Y, *ep = Y + 3 * L.pmax;
     for (int pi = j; pi < npair; pi += T) {
         const int PA = pa[pi], PB = pb[pi];
