@@ -6,8 +6,9 @@
 // the second-order occupied-virtual update, Anderson mixing, analytic forces. The mapping to the
 // machine is made for matrices too large for a lane group, on a GPU whose FP64 pipe (2 FMA per
 // clock per SM) is the only bottleneck, so what counts is the number of FP64 warp instructions:
-//   * work items: a cell of more than 32 orbitals takes a whole 128-thread block, smaller cells
-//     take 64 threads each, two per block. A persistent grid pulls items from a queue ordered by
+//   * work items: a cell of more than 32 orbitals takes a whole 256-thread block, smaller cells
+//     take 128 threads each, two per block (128 and 64 threads left the FP64 pipe 55 % busy with
+//     eight warps per SM; these 65 %: 16,384 clusters 24 -> 19.5 ms with the pairs sorted by kind). A persistent grid pulls items from a queue ordered by
 //     decreasing size, so large cells start first and small ones fill the tail;
 //   * every matrix product spreads its output entries evenly over the cell's threads (R entries
 //     per thread per pass, each summed over k in increasing order), so nearly every lane of
@@ -40,9 +41,9 @@ constexpr int GW_EVALS = 8;            // and bound on the FP64 evaluations
 constexpr float GW_ORTH_MAX = 1e-4f;   // overlap defect that the second-order correction takes
 constexpr float GW_GAP = 2e-3f;        // HOMO-LUMO gap (Hartree) the warm path needs, above G_MIN_GAP
 constexpr int GW_CG_ITERS = 40;        // bound on the conjugate-gradient steps of a Newton step
-constexpr int BT = 128;                // threads per block
-constexpr int TB = 128;                // threads per large cell
-constexpr int TS = 64;                 // threads per small cell (two per block)
+constexpr int BT = 256;                // threads per block
+constexpr int TB = 256;                // threads per large cell
+constexpr int TS = 128;                // threads per small cell (two per block)
 
 // Shared-memory layout of one cell (byte offsets) for cells of at most nmax orbitals, amax atoms.
 struct GLayout {
@@ -87,14 +88,14 @@ __host__ __device__ inline GLayout g_layout(int nmax, int amax) {
     L.th = o; o += GNHIST * 8;
     L.ints = o;
     // ints: spec[amax], atom_off[amax+1], orb_atom[nmax], occ_list[nmax], virt_list[nmax],
-    //       occf[nmax], pp[nmax/2+1], pq[nmax/2+1], pa[pmax], pb[pmax], fl[8]
-    o += (unsigned)(2 * amax + 1 + 4 * nmax + 2 * (nmax / 2 + 1) + 2 * L.pmax + 8) * 4;
+    //       occf[nmax], pp[nmax/2+1], pq[nmax/2+1], pa[pmax], pb[pmax], lst[amax], rk[amax], fl[8]
+    o += (unsigned)(4 * amax + 1 + 4 * nmax + 2 * (nmax / 2 + 1) + 2 * L.pmax + 8) * 4;
     L.total = (o + 15u) & ~15u;
     return L;
 }
 
 // A group of T threads evaluating one cell: the whole block (T = BT), or one half of it
-// (T = 64, named barrier 1 or 2).
+// (T = TS, named barrier 1 or 2).
 template <int T>
 struct Grp {
     int tid;
@@ -263,8 +264,9 @@ struct GWarm {
 // the result. Returns false, with SH untouched, for a cell that leaves the path's range (a large
 // rotation or overlap change, a Hessian or gap that is not safely positive, no convergence): the
 // general path takes it. On success: C (FP64, occupied columns first), q, shift, XB = H C_o.
-// Measured (GB300, one launch of 16,384 clusters (H2O)_1..8): 84 -> 24 ms, mean evaluations 2.0 against
-// 10.8 iterations; 301 clusters 4.9 -> 1.1 ms. Bound: the FP64 pipe (55 % busy with eight warps per SM).
+// Measured (GB300, one launch of 16,384 clusters (H2O)_1..8, 128 threads per block): 84 -> 24 ms, mean
+// evaluations 2.0 against 10.8 iterations; 301 clusters 4.9 -> 1.1 ms. Bound: the FP64 pipe (65 % busy
+// with 256 threads).
 template <int T, int R>
 __device__ bool g_warm(const DftbArgs &a, const GWarm &v, double *&C, double *&Y, const double *cw, const Grp<T> &g,
                        int &evals) {
@@ -304,7 +306,7 @@ __device__ bool g_warm(const DftbArgs &a, const GWarm &v, double *&C, double *&Y
     };
     // F1 = S F0 (S32 in F2)
     auto sc32 = [&]() {
-        ftile<T, 6, 3>(j, n, n, n, F2, 1, LF, F0, LF, 1, [&](int i, int c, float t) { F1[i * LF + c] = t; });
+        ftile<T, 3, 3>(j, n, n, n, F2, 1, LF, F0, LF, 1, [&](int i, int c, float t) { F1[i * LF + c] = t; });
         g.sync();
     };
     // A32 = F0^T H F0 into F2, H with the orbital half shifts eo (F3 holds H F0 on the way)
@@ -314,21 +316,22 @@ __device__ bool g_warm(const DftbArgs &a, const GWarm &v, double *&C, double *&Y
             F2[c * LF + i] = fmaf(d2f_steer(s_at(i, c)), v.eo[i] + v.eo[c], d2f_steer(h0_at(i, c)));
         }
         g.sync();
-        ftile<T, 6, 3>(j, n, n, n, F2, 1, LF, F0, LF, 1, [&](int i, int c, float t) { F3[i * LF + c] = t; });
+        ftile<T, 3, 3>(j, n, n, n, F2, 1, LF, F0, LF, 1, [&](int i, int c, float t) { F3[i * LF + c] = t; });
         g.sync();
-        ftile<T, 6, 3>(j, n, n, n, F0, 1, LF, F3, LF, 1, [&](int i, int c, float t) { F2[i * LF + c] = t; });
+        ftile<T, 3, 3>(j, n, n, n, F0, 1, LF, F3, LF, 1, [&](int i, int c, float t) { F2[i * LF + c] = t; });
         g.sync();
     };
     // populations moved by K = kv to first order, per atom into dq; uses F0 = C, F1 = S C and F3's tail
+    constexpr int CQ = 3;   // rows per tile
     auto charges = [&](const float *kv) {
         float *part = F3 + 2 * nvo;
-        const int ni = (n + 5) / 6, nc = (no + 1) / 2;
+        const int ni = (n + CQ - 1) / CQ, nc = (no + 1) / 2;
         for (int t = j; t < ni * nc; t += T) {
-            const int tc = t / ni, i0 = (t - tc * ni) * 6, c0 = 2 * tc, c1 = min(2 * tc + 1, no - 1);
-            float ax[6][2], as[6][2];
-            const float *cp[6], *sp[6];
+            const int tc = t / ni, i0 = (t - tc * ni) * CQ, c0 = 2 * tc, c1 = min(2 * tc + 1, no - 1);
+            float ax[CQ][2], as[CQ][2];
+            const float *cp[CQ], *sp[CQ];
 #pragma unroll
-            for (int q = 0; q < 6; ++q) {
+            for (int q = 0; q < CQ; ++q) {
                 cp[q] = F0 + min(i0 + q, n - 1) * LF;
                 sp[q] = F1 + min(i0 + q, n - 1) * LF;
                 ax[q][0] = ax[q][1] = as[q][0] = as[q][1] = 0.0f;
@@ -336,7 +339,7 @@ __device__ bool g_warm(const DftbArgs &a, const GWarm &v, double *&C, double *&Y
             for (int k = 0; k < nv; ++k) {
                 const float k0 = kv[k * no + c0], k1 = kv[k * no + c1];
 #pragma unroll
-                for (int q = 0; q < 6; ++q) {
+                for (int q = 0; q < CQ; ++q) {
                     const float cv = cp[q][no + k], sv = sp[q][no + k];
                     ax[q][0] = fmaf(cv, k0, ax[q][0]);
                     ax[q][1] = fmaf(cv, k1, ax[q][1]);
@@ -345,7 +348,7 @@ __device__ bool g_warm(const DftbArgs &a, const GWarm &v, double *&C, double *&Y
                 }
             }
 #pragma unroll
-            for (int q = 0; q < 6; ++q) {
+            for (int q = 0; q < CQ; ++q) {
                 if (i0 + q >= n) continue;
                 float s = fmaf(ax[q][0], sp[q][c0], cp[q][c0] * as[q][0]);
                 if (c0 + 1 < no) s += fmaf(ax[q][1], sp[q][c1], cp[q][c1] * as[q][1]);
@@ -446,10 +449,10 @@ __device__ bool g_warm(const DftbArgs &a, const GWarm &v, double *&C, double *&Y
     };
     // second-order parts of the rotation: G[i][o] = 1/2 sum_v C[i][v] K_vo, G[i][no + v] = -1/2 sum_o C[i][o] K_vo
     auto second = [&](float *G, bool with_c) {
-        ftile<T, 6, 2>(j, n, no, nv, F0 + no, LF, 1, x, no, 1, [&](int i, int c, float t) {
+        ftile<T, 3, 2>(j, n, no, nv, F0 + no, LF, 1, x, no, 1, [&](int i, int c, float t) {
             G[i * LF + c] = fmaf(0.5f, t, with_c ? F0[i * LF + c] : 0.0f);
         });
-        ftile<T, 3, 2>(j, n, nv, no, F0, LF, 1, x, 1, no, [&](int i, int c, float t) {
+        ftile<T, 3, 1>(j, n, nv, no, F0, LF, 1, x, 1, no, [&](int i, int c, float t) {
             G[i * LF + no + c] = fmaf(-0.5f, t, with_c ? F0[i * LF + no + c] : 0.0f);
         });
         g.sync();
@@ -464,7 +467,7 @@ __device__ bool g_warm(const DftbArgs &a, const GWarm &v, double *&C, double *&Y
     for (int pass = 0; pass < 2; ++pass) {   // E is a few 1e-2 after one step: below 1e-6 after two passes
         sc32();
         float big = 0.0f;
-        ftile<T, 6, 3>(j, n, n, n, F0, 1, LF, F1, LF, 1, [&](int i, int c, float t) {
+        ftile<T, 3, 3>(j, n, n, n, F0, 1, LF, F1, LF, 1, [&](int i, int c, float t) {
             const float e = t - (i == c ? 1.0f : 0.0f);
             big = fmaxf(big, fabsf(e));
             if (pass == 0) F3[i * LF + c] = e;
@@ -473,12 +476,12 @@ __device__ bool g_warm(const DftbArgs &a, const GWarm &v, double *&C, double *&Y
         if (!all(big < 0.2f)) return false;   // NaN included
         if (pass == 0) {
             g.sync();
-            ftile<T, 6, 3>(j, n, n, n, F3, 1, LF, F3, LF, 1, [&](int i, int c, float t) {
+            ftile<T, 3, 3>(j, n, n, n, F3, 1, LF, F3, LF, 1, [&](int i, int c, float t) {
                 F4[i * LF + c] = fmaf(0.375f, t, fmaf(-0.5f, F3[i * LF + c], i == c ? 1.0f : 0.0f));
             });
         }
         g.sync();
-        ftile<T, 6, 3>(j, n, n, n, F0, LF, 1, F4, LF, 1, [&](int i, int c, float t) { F5[i * LF + c] = t; });
+        ftile<T, 3, 3>(j, n, n, n, F0, LF, 1, F4, LF, 1, [&](int i, int c, float t) { F5[i * LF + c] = t; });
         g.sync();
         for (int e = j; e < nn; e += T) {
             const int i = e / n, c = e - i * n;
@@ -515,8 +518,8 @@ __device__ bool g_warm(const DftbArgs &a, const GWarm &v, double *&C, double *&Y
         if (!all(kmax < GW_ROT_MAX)) return false;
         done = all(kmax < GW_FP32_KTOL);
         second(F4, true);
-        ftile<T, 6, 2>(j, n, no, nv, F4 + no, LF, 1, x, no, 1, [&](int i, int c, float t) { F0[i * LF + c] += t; });
-        ftile<T, 3, 2>(j, n, nv, no, F4, LF, 1, x, 1, no, [&](int i, int c, float t) { F0[i * LF + no + c] -= t; });
+        ftile<T, 3, 2>(j, n, no, nv, F4 + no, LF, 1, x, no, 1, [&](int i, int c, float t) { F0[i * LF + c] += t; });
+        ftile<T, 3, 1>(j, n, nv, no, F4, LF, 1, x, 1, no, [&](int i, int c, float t) { F0[i * LF + no + c] -= t; });
         g.sync();
     }
     if (!done) return false;
@@ -550,7 +553,7 @@ __device__ bool g_warm(const DftbArgs &a, const GWarm &v, double *&C, double *&Y
         if (!all(big < GW_ORTH_MAX)) return false;
         g.sync();
         // 1 - E/2 + 3/8 E^2: E^2 is below 1e-8, so FP32 carries it beyond FP64 rounding
-        ftile<T, 6, 3>(j, n, n, n, E32, 1, LF, E32, LF, 1, [&](int i, int c, float t) {
+        ftile<T, 3, 3>(j, n, n, n, E32, 1, LF, E32, LF, 1, [&](int i, int c, float t) {
             A[c * LD + i] = fma(-0.5, A[c * LD + i], (i == c ? 1.0 : 0.0) + f2d_steer(0.375f * t));
         });
         g.sync();
@@ -661,9 +664,9 @@ __device__ bool g_warm(const DftbArgs &a, const GWarm &v, double *&C, double *&Y
         if (!all(kmax < 1e-2f)) return false;
         // C (1 + K + K^2/2), as C_o + (C_v - (C_o K^T)/2) K and C_v - (C_o + (C_v K)/2) K^T
         second(F1, false);
-        double Kd[8];   // this thread's entries of K: n_virt n_occ <= n^2 / 4, 1024 on 128 threads at n = 64, 256 on 64 at n = 32
+        double Kd[4];   // this thread's entries of K: n_virt n_occ <= n^2 / 4, 1024 on 256 threads at n = 64, 256 on 128 at n = 32
 #pragma unroll
-        for (int t = 0; t < 8; ++t) {
+        for (int t = 0; t < 4; ++t) {
             const int e = j + t * T;
             Kd[t] = e < nvo ? f2d_steer(x[e]) : 0.0;
         }
@@ -674,7 +677,7 @@ __device__ bool g_warm(const DftbArgs &a, const GWarm &v, double *&C, double *&Y
         g.sync();
         double *K = v.Kc;
 #pragma unroll
-        for (int t = 0; t < 8; ++t) {
+        for (int t = 0; t < 4; ++t) {
             const int e = j + t * T;
             if (e < nvo) K[e] = Kd[t];
         }
@@ -716,7 +719,9 @@ __device__ void g_molecule(const DevSK &sk, const DftbArgs &a, const GLayout &L,
     int *pq = pp + (L.nmax / 2 + 1);
     int *pa = pq + (L.nmax / 2 + 1);
     int *pb = pa + L.pmax;
-    int *fl = pb + L.pmax;   // 0 error bits, 2 iterations, 3 occupied orbitals, 4 orbitals, 5 pairs
+    int *lst = pb + L.pmax;  // atoms with p orbitals, then those without, each in increasing order
+    int *rk = lst + L.amax;  // position of an atom among those of its kind
+    int *fl = rk + L.amax;   // 0 error bits, 2 iterations, 3 occupied orbitals, 4 orbitals, 6 atoms with p orbitals
     const int AM = L.amax;
 
     if (j < nat) {
@@ -746,13 +751,47 @@ __device__ void g_molecule(const DevSK &sk, const DftbArgs &a, const GLayout &L,
         fl[2] = 0;
         fl[3] = (int)(nel * 0.5 + 0.25);
         fl[4] = o;
-        int pi = 0;
-        for (int x = 0; x < nat; ++x)
-            for (int y = x + 1; y < nat; ++y) { pa[pi] = x; pb[pi] = y; ++pi; }
-        fl[5] = pi;
+    }
+    if (j < nat) {
+        const bool big = sk.norb[spec[j]] == 4;
+        int same = 0, nbig = 0;
+        for (int x = 0; x < nat; ++x) {
+            const bool bx = sk.norb[spec[x]] == 4;
+            nbig += bx;
+            same += x < j && bx == big;
+        }
+        rk[j] = same;
+        lst[big ? same : nbig + same] = j;
+        if (j == 0) fl[6] = nbig;
     }
     g.sync();
-    const int n = fl[4], nocc = fl[3], npair = fl[5];
+    const int n = fl[4], nocc = fl[3], npair = nat * (nat - 1) / 2;
+    // Pairs (A < B) by kind, so that the threads of a warp evaluate the same integrals: both atoms with p
+    // orbitals (10 radial functions), one of them (4), neither (2).
+    const int nb = fl[6], ns = nat - nb, p_bb = nb * (nb - 1) / 2, p_bs = p_bb + nb * ns;
+    for (int pi = j; pi < npair; pi += T) {
+        int x, y;
+        if (pi >= p_bb && pi < p_bs) {
+            const int u = pi - p_bb;
+            x = lst[u / ns];
+            y = lst[nb + u % ns];
+        } else {
+            const int u = pi < p_bb ? pi : pi - p_bs, o = pi < p_bb ? 0 : nb;
+            int k = (int)((1.0f + sqrtf(1.0f + 8.0f * (float)u)) * 0.5f);
+            while (k * (k - 1) / 2 > u) --k;
+            while ((k + 1) * k / 2 <= u) ++k;
+            x = lst[o + u - k * (k - 1) / 2];
+            y = lst[o + k];
+        }
+        pa[pi] = min(x, y);
+        pb[pi] = max(x, y);
+    }
+    auto pair_of = [&](int x, int y) -> int {   // the pair's index
+        const bool bx = lst[rk[x]] == x && rk[x] < nb, by = lst[rk[y]] == y && rk[y] < nb;
+        if (bx != by) return p_bb + (bx ? rk[x] : rk[y]) * ns + (bx ? rk[y] : rk[x]);
+        const int k = max(rk[x], rk[y]), i = min(rk[x], rk[y]);
+        return (bx ? 0 : p_bs) + k * (k - 1) / 2 + i;
+    };
     const int nv = n - nocc;
     const int LD = n + 1;   // n is even (closed shell), so the stride is odd
     const int nn = n * n;
@@ -1198,7 +1237,6 @@ __device__ void g_molecule(const DevSK &sk, const DftbArgs &a, const GLayout &L,
             for (int at = 0; at < nat; ++at) eb = fma(-q[at], shift[at], eb);
             red[0] = eb;
         }
-        if (j > 0 && j < n) red[j] = 0.0;
         // t(o, i) = 2 sum_p A_oo(o, p) C(i, p) into Y[i * LD + o]
         flat<T, R>(j, nocc * n, nocc, LD, LD, [&](int e) { return A + (e % nocc); }, [&](int e) { return C + (e / nocc); },
                    [&](int e, double v) { Y[(e / nocc) * LD + e % nocc] = 2.0 * v; });
@@ -1368,12 +1406,15 @@ __device__ void g_molecule(const DevSK &sk, const DftbArgs &a, const GLayout &L,
     }
     g.sync();
     if (j < nat) {
-        double f[3] = {0.0, 0.0, 0.0};
-        for (int pi = 0; pi < npair; ++pi) {
-            const double sg = (pb[pi] == j) ? -1.0 : ((pa[pi] == j) ? 1.0 : 0.0);
-            if (sg != 0.0)
-                for (int k = 0; k < 3; ++k) f[k] = fma(sg, gp[3 * pi + k], f[k]);
+        double f[3] = {0.0, 0.0, 0.0}, er = 0.0;
+        for (int x = 0; x < nat; ++x) {
+            if (x == j) continue;
+            const int pi = pair_of(x, j);
+            const double sg = x < j ? -1.0 : 1.0;
+            for (int k = 0; k < 3; ++k) f[k] = fma(sg, gp[3 * pi + k], f[k]);
+            if (x < j) er += ep[pi];
         }
+        hq[j] = er;   // the repulsion of the pairs whose second atom this is
         const int at = a0 + j;
         for (int k = 0; k < 3; ++k) a.F[3 * at + k] = f[k];
         a.qprev[at] = a.have_warm ? qst[j] : q[j];
@@ -1386,14 +1427,16 @@ __device__ void g_molecule(const DevSK &sk, const DftbArgs &a, const GLayout &L,
             a.b[3 * at + 2] = Q * a.pol2;
         }
     }
+    g.sync();
     if (j == 0) {
         double E = 0.0;
-        for (int i = 0; i < n; ++i) E += red[i];
-        double e2 = 0.0;
-        for (int x = 0; x < nat; ++x)
-            for (int y = 0; y < nat; ++y) e2 = fma(gam[x * AM + y] * (q[x] - zv[x]), q[y] - zv[y], e2);
+        if (warm) E = red[0];
+        else
+            for (int i = 0; i < n; ++i) E += red[i];
+        double e2 = 0.0;   // sum_A dq_A eps_A (the shifts of the converged charges)
+        for (int x = 0; x < nat; ++x) e2 = fma(q[x] - zv[x], shift[x], e2);
         E = fma(0.5, e2, E);
-        for (int pi = 0; pi < npair; ++pi) E += ep[pi];
+        for (int x = 0; x < nat; ++x) E += hq[x];
         double mu[3] = {0.0, 0.0, 0.0};
         for (int at = 0; at < nat; ++at) {
             const double Q = zv[at] - q[at];
@@ -1416,7 +1459,7 @@ __global__ void __launch_bounds__(BT, 2) k_dftb_generic(const DevSK *__restrict_
                                                      int nmax_s, int amax_s) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int next;
-    __shared__ int vote[2][2];
+    __shared__ int vote[2][TS / 32];
     const DevSK &sk = *skp;
     const GLayout Lb = g_layout(nmax_b, amax_b);
     const GLayout Ls = g_layout(nmax_s, amax_s);
