@@ -396,8 +396,8 @@ cudaError_t enqueue_steps(cavmd_ctx *c, int64_t n, int64_t first_step) {
 // The context's own state is not touched.
 int autotune(cavmd_ctx *c) {
     if (c->periodic) {
-        c->tuning = c->pplan.nk > 0 ? "k_dftb_periodic_kg: one 256-thread block per cell, one per SM (no candidates)"
-                                    : "k_dftb_periodic: one 256-thread block per cell, two per SM (no candidates)";
+        c->tuning = c->pplan.nk > 0 ? "k_dftb_periodic_kg: clusters of " + std::to_string(c->pplan.cluster) + " 256-thread blocks, one cell each (no candidates)"
+                                    : std::string("k_dftb_periodic: one 256-thread block per cell, two per SM (no candidates)");
         return CAVMD_OK;
     }
     const int NA = c->n_atoms, N = c->N;
@@ -993,10 +993,11 @@ int build_context(cavmd_ctx *c, const cavmd_system *sys, const cavmd_sk_tables *
         }
         int nsm = 0;
         CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device));
-        pp.blocks = std::max(1, std::min(N, (nk > 0 ? 1 : 2) * nsm));
+        CK(prepare_dftb_periodic());
+        CK(plan_dftb_periodic_launch(pp, N, nsm));
         AL(pp.d_img, img.size());
         AL(pp.d_gw, gw.size());
-        AL(pp.work, pbc_workspace_doubles(pp.nmax, pp.amax, pp.n_g, nk) * (size_t)pp.blocks);
+        AL(pp.work, pbc_workspace_doubles(pp.nmax, pp.amax, pp.n_g, nk, pp.cluster) * (size_t)pp.blocks);
         if (nk > 0) {
             AL(pp.d_kpt, kpts.size());
             CK(cudaMemcpyAsync(pp.d_kpt, kpts.data(), sizeof(double) * kpts.size(), cudaMemcpyHostToDevice, st));
@@ -1005,7 +1006,6 @@ int build_context(cavmd_ctx *c, const cavmd_system *sys, const cavmd_sk_tables *
         CK(cudaMemcpyAsync(pp.d_gw, gw.data(), sizeof(double) * gw.size(), cudaMemcpyHostToDevice, st));
         AL(c->d_Coff, N);
         CK(cudaMemcpyAsync(c->d_Coff, coff.data(), sizeof(long long) * N, cudaMemcpyHostToDevice, st));
-        CK(prepare_dftb_periodic());
         CK(cudaStreamSynchronize(st));   // the host vectors must outlive the copies
     }
 

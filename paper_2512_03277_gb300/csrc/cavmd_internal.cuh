@@ -248,6 +248,7 @@ struct GenericPlan {
 void plan_dftb_generic(const int *cell_offset, const int *species, const int *norb_of_elem, int n_cells,
                        int n_disp_per_atom, GenericPlan &p, std::vector<int2> &items,
                        std::vector<int2> &disp_items);
+const void *dftb_generic_kernel_r2();   // the variant with two product entries per thread
 cudaError_t prepare_dftb_generic(GenericPlan &p);   // kernel attribute and occupancy, once per plan
 cudaError_t launch_dftb_generic(const DevSK *sk_dev, const DftbArgs &a, const GenericPlan &p, cudaStream_t st);
 // Plan of the Gamma-point SCC-DFTB launch over periodic cells (one lattice for all cells).
@@ -256,18 +257,21 @@ struct PbcPlan {
     double alpha, bg, self_e, r_real;     // Ewald splitting, background and self terms, real-space cutoff
     int n_img, n_img_sk, n_g;             // lattice translations (by length; the first n_img_sk reach
                                           // r_cut); half-space reciprocal vectors
-    int nmax, amax, blocks;               // largest cell; persistent blocks (2 per SM, k-grid 1)
+    int nmax, amax;                       // largest cell
+    int blocks, cluster;                  // cells in flight; blocks that share a cell (k-grid; else 1)
     double *d_img, *d_gw;                 // device: [n_img][3], [n_g][4] (G, 2 w_G)
     double *work;                         // device: per-block workspaces
     int nk;                               // k-grid: irreducible k-points (0: Gamma point only)
     double *d_kpt;                        // device: [nk][4] fractional k and weight
 };
-size_t pbc_workspace_doubles(int nmax, int amax, int n_g, int nk);
+size_t pbc_workspace_doubles(int nmax, int amax, int n_g, int nk, int cluster);
+const void *pbc_kg_small();   // the k-grid kernels (problems up to 256 and up to 512 wide)
+const void *pbc_kg_large();
 std::vector<double> pbc_kpoints(const int *kgrid);
-size_t pbc_smem(bool kgrid);
 void plan_dftb_periodic(const double *lat, double r_cut, PbcPlan &p, std::vector<double> &img,
                         std::vector<double> &gw);
-cudaError_t prepare_dftb_periodic();
+cudaError_t prepare_dftb_periodic();   // kernel attributes, before plan_dftb_periodic_launch
+cudaError_t plan_dftb_periodic_launch(PbcPlan &p, int n_cells, int n_sm);
 cudaError_t launch_dftb_periodic(const DevSK *sk_dev, const DftbArgs &a, const PbcPlan &p, cudaStream_t st);
 // b_j = dM/dr_j from the displaced dipoles (forward or central differences)
 cudaError_t launch_born_assemble(int n_cells, const int *cell_offset, const double *M_cell,
