@@ -268,7 +268,7 @@ struct GWarm {
 // evaluations 2.0 against 10.8 iterations; 301 clusters 4.9 -> 1.1 ms. Bound: the FP64 pipe (65 % busy
 // with 256 threads).
 template <int T>
-__device__ __noinline__ bool g_warm(const DftbArgs &a, const GWarm &v, double *&C, double *&Y, const double *cw, const Grp<T> &g,
+__device__ bool g_warm(const DftbArgs &a, const GWarm &v, double *&C, double *&Y, const double *cw, const Grp<T> &g,
                        int &evals) {
     const int j = g.tid;
     const int n = v.n, no = v.nocc, nv = n - no, nat = v.nat, LD = n + 1, LF = n + 1, nn = n * n, nvo = nv * no;

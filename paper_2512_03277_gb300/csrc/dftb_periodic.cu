@@ -227,19 +227,22 @@ cudaError_t launch_dftb_periodic(const DevSK *sk_dev, const DftbArgs &a, const P
     const long long items = a.n_disp > 0 ? (long long)a.n_cells * (a.fd_central ? 6 : 3) * p.amax : a.n_cells;
     const int groups = (int)std::min<long long>(items, p.blocks);
     if (p.nk > 0) {
+        // a cold start (the general path, one block per cell) takes the wider kernel's registers
+        const bool cold = !a.have_warm;
+        if (cold) d.cluster = 1;
         cudaLaunchConfig_t cfg = {};
         cudaLaunchAttribute at[1];
-        cfg.gridDim = dim3(groups * p.cluster);
+        cfg.gridDim = dim3(groups * d.cluster);
         cfg.blockDim = dim3(PT);
-        cfg.dynamicSmemBytes = kg_smem(p.nmax);
+        cfg.dynamicSmemBytes = kg_smem(cold ? PNMAX : p.nmax);
         cfg.stream = st;
         at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = p.cluster;
+        at[0].val.clusterDim.x = d.cluster;
         at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
         cfg.attrs = at;
         cfg.numAttrs = 1;
         void *args[] = {(void *)&sk_dev, (void *)&a, (void *)&d};
-        return cudaLaunchKernelExC(&cfg, kg_kernel(p.nmax), args);
+        return cudaLaunchKernelExC(&cfg, kg_kernel(cold ? PNMAX : p.nmax), args);
     }
     k_dftb_periodic<<<groups, PT, sizeof(PShared), st>>>(sk_dev, a, d);
     return cudaGetLastError();

@@ -76,9 +76,10 @@ struct PSharedT {
     double th[PHIST];
     double gred[PT / 32][3];
     int spec[PAMAX], atom_off[PAMAX + 1], orb_atom[PNMAX];
+    int lst[PAMAX];              // atoms with p orbitals, then those without
     int occ_list[PN], virt_list[PN], occf[PN];
     int pp[PN / 2], pq[PN / 2];
-    int fl[8];                   // 0 error bits, 1 n, 2 iterations, 3 occupied orbitals
+    int fl[8];                   // 0 error bits, 1 n, 2 iterations, 3 occupied orbitals, 5 atoms with p orbitals
     int vote[PT / 32];
 };
 using PShared = PSharedT<PNMAX>;
@@ -909,6 +910,54 @@ __device__ __noinline__ bool p_warm(const DftbArgs &a, const PbcDev &pl, SH &sh,
     return false;
 }
 
+// Calls f(im) for the lattice images (of the first n_img) whose distance from the wrapped separation dw may be
+// below sqrt(r2max), in increasing order. Each thread first marks its own images in FP32 (with a margin;
+// f applies the exact test) and then visits those: the threads of a warp reach different images, and a plain
+// loop would run f's long body for every image that any of them reaches.
+template <class F>
+__device__ __forceinline__ void pbc_images(const PbcDev &pl, const double *dw, int n_img, double r2max, F f) {
+    const float x = d2f_steer(dw[0]), y = d2f_steer(dw[1]), z = d2f_steer(dw[2]);
+    const float lim = fmaf(d2f_steer(r2max), 1.0001f, 1e-2f);
+    for (int base = 0; base < n_img; base += 32) {
+        unsigned mask = 0u;
+        const int end = min(32, n_img - base);
+        for (int b = 0; b < end; ++b) {
+            const double *t = pl.img + 3 * (base + b);
+            const float u = x + d2f_steer(t[0]), v = y + d2f_steer(t[1]), w = z + d2f_steer(t[2]);
+            if (fmaf(u, u, fmaf(v, v, w * w)) < lim) mask |= 1u << b;
+        }
+        while (mask) {
+            const int b = __ffs(mask) - 1;
+            mask &= mask - 1u;
+            f(base + b);
+        }
+    }
+}
+
+// Pair A <= B number t of a cell, by kind: both atoms with p orbitals, one of them, neither, then each atom
+// with its own images. The threads of a warp then evaluate the same radial functions.
+template <class SH>
+__device__ __forceinline__ void pbc_pair(const SH &sh, int nat, int t, int &A, int &B) {
+    const int nb = sh.fl[5], ns = nat - nb, p_bb = nb * (nb - 1) / 2, p_bs = p_bb + nb * ns, p_all = nat * (nat - 1) / 2;
+    int x, y;
+    if (t >= p_all) {
+        x = y = t - p_all;
+    } else if (t >= p_bb && t < p_bs) {
+        const int u = t - p_bb;
+        x = sh.lst[u / ns];
+        y = sh.lst[nb + u % ns];
+    } else {
+        const int u = t < p_bb ? t : t - p_bs, o = t < p_bb ? 0 : nb;
+        int k = (int)((1.0f + sqrtf(1.0f + 8.0f * (float)u)) * 0.5f);
+        while (k * (k - 1) / 2 > u) --k;
+        while ((k + 1) * k / 2 <= u) ++k;
+        x = sh.lst[o + u - k * (k - 1) / 2];
+        y = sh.lst[o + k];
+    }
+    A = min(x, y);
+    B = max(x, y);
+}
+
 // One cell, or (disp_k >= 0) one finite-difference copy of it: atom disp_k / 3 (central: disp_k / 6)
 // moved along x, y or z by +h (central: +h and -h in turn), warm started from the cell's converged
 // basis in a private copy, and only its dipole written (M_disp, the layout of the water kernels).
@@ -966,6 +1015,17 @@ __device__ void p_cell(const DevSK &sk, const DftbArgs &a, const PbcDev &pl, SH 
         sh.fl[2] = 0;
         sh.fl[3] = (int)(nel * 0.5 + 0.25);
     }
+    if (j < nat) {
+        const bool big = sk.norb[sh.spec[j]] == 4;
+        int same = 0, nbig = 0;
+        for (int x = 0; x < nat; ++x) {
+            const bool bx = sk.norb[sh.spec[x]] == 4;
+            nbig += bx;
+            same += x < j && bx == big;
+        }
+        sh.lst[big ? same : nbig + same] = j;
+        if (j == 0) sh.fl[5] = nbig;
+    }
     __syncthreads();
     const int n = sh.fl[1], nocc = sh.fl[3];
     const int nv = n - nocc, nn = n * n;
@@ -1008,8 +1068,9 @@ __device__ void p_cell(const DevSK &sk, const DftbArgs &a, const PbcDev &pl, SH 
                 S[e] = s;
             }
             __syncthreads();
-            for (int t = j; t < nat * (nat + 1) / 2; t += PT) {   // pairs A <= B, packed by A
-                const int A = lower_col(t, nat), B = A + (t - (A * nat - A * (A - 1) / 2));
+            for (int t = j; t < nat * (nat + 1) / 2; t += PT) {   // pairs A <= B, by kind
+                int A, B;
+                pbc_pair(sh, nat, t, A, B);
                 const int eA = sh.spec[A], eB = sh.spec[B];
                 const int oA = sh.atom_off[A], oB = sh.atom_off[B];
                 const int na = sk.norb[eA], nb = sk.norb[eB];
@@ -1022,18 +1083,18 @@ __device__ void p_cell(const DevSK &sk, const DftbArgs &a, const PbcDev &pl, SH 
                 double g_re = 0.0, g_sr = 0.0;
                 const double c2 = sk.gamma_c2[eA][eB];
                 if (first) {
-                    for (int im = 0; im < pl.n_img; ++im) {   // real-space Ewald sum
+                    pbc_images(pl, dw, pl.n_img, pl.r_real2, [&](int im) {   // real-space Ewald sum
                         const double x0 = dw[0] + pl.img[3 * im], x1 = dw[1] + pl.img[3 * im + 1], x2 = dw[2] + pl.img[3 * im + 2];
                         const double r2 = fma(x0, x0, fma(x1, x1, x2 * x2));
-                        if (!(r2 < pl.r_real2) || r2 == 0.0) continue;
+                        if (!(r2 < pl.r_real2) || r2 == 0.0) return;
                         const double ir = rsqrt_nr(r2);
                         g_re = fma(erfc(pl.alpha * (r2 * ir)), ir, g_re);
-                    }
+                    });
                 }
-                for (int im = 0; im < pl.n_img_sk; ++im) {   // images within r_cut
+                pbc_images(pl, dw, pl.n_img_sk, rc2, [&](int im) {   // images within r_cut
                     const double x0 = dw[0] + pl.img[3 * im], x1 = dw[1] + pl.img[3 * im + 1], x2 = dw[2] + pl.img[3 * im + 2];
                     const double r2 = fma(x0, x0, fma(x1, x1, x2 * x2));
-                    if (!(r2 < rc2) || r2 == 0.0) continue;
+                    if (!(r2 < rc2) || r2 == 0.0) return;
                     const double ir = rsqrt_nr(r2);
                     const double r = r2 * ir;
                     const double e[3] = {x0 * ir, x1 * ir, x2 * ir};
@@ -1080,7 +1141,7 @@ __device__ void p_cell(const DevSK &sk, const DftbArgs &a, const PbcDev &pl, SH 
                         cutoff_fn(r, sk, fc, dfc);
                         g_sr = fma(rsqrt_nr(r2 + c2) - ir, fc, g_sr);
                     }
-                }
+                });
                 // complex block z (mu of A, nu of B) at row oA + mu, column oB + nu of [[Re, -Im], [Im, Re]],
                 // and its Hermitian transpose; a block of an atom with its own images is Hermitian,
                 // written as the mean of z and the conjugate transpose
@@ -1132,8 +1193,9 @@ __device__ void p_cell(const DevSK &sk, const DftbArgs &a, const PbcDev &pl, SH 
             S[e] = s;
         }
         __syncthreads();
-        for (int t = j; t < nat * (nat + 1) / 2; t += PT) {   // pairs A <= B, packed by A
-            const int A = lower_col(t, nat), B = A + (t - (A * nat - A * (A - 1) / 2));
+        for (int t = j; t < nat * (nat + 1) / 2; t += PT) {   // pairs A <= B, by kind
+            int A, B;
+                pbc_pair(sh, nat, t, A, B);
             const int eA = sh.spec[A], eB = sh.spec[B];
             const int oA = sh.atom_off[A], oB = sh.atom_off[B];
             const int na = sk.norb[eA], nb = sk.norb[eB];
@@ -1146,17 +1208,17 @@ __device__ void p_cell(const DevSK &sk, const DftbArgs &a, const PbcDev &pl, SH 
             double g_re = 0.0, g_sr = 0.0;
             const double c2 = sk.gamma_c2[eA][eB];
             const double rc2 = sk.r_cut * sk.r_cut;
-            for (int im = 0; im < pl.n_img; ++im) {   // real-space Ewald sum
+            pbc_images(pl, dw, pl.n_img, pl.r_real2, [&](int im) {   // real-space Ewald sum
                 const double x0 = dw[0] + pl.img[3 * im], x1 = dw[1] + pl.img[3 * im + 1], x2 = dw[2] + pl.img[3 * im + 2];
                 const double r2 = fma(x0, x0, fma(x1, x1, x2 * x2));
-                if (!(r2 < pl.r_real2) || r2 == 0.0) continue;
+                if (!(r2 < pl.r_real2) || r2 == 0.0) return;
                 const double ir = rsqrt_nr(r2);
                 g_re = fma(erfc(pl.alpha * (r2 * ir)), ir, g_re);
-            }
-            for (int im = 0; im < pl.n_img_sk; ++im) {   // images within r_cut
+            });
+            pbc_images(pl, dw, pl.n_img_sk, rc2, [&](int im) {   // images within r_cut
                 const double x0 = dw[0] + pl.img[3 * im], x1 = dw[1] + pl.img[3 * im + 1], x2 = dw[2] + pl.img[3 * im + 2];
                 const double r2 = fma(x0, x0, fma(x1, x1, x2 * x2));
-                if (!(r2 < rc2) || r2 == 0.0) continue;
+                if (!(r2 < rc2) || r2 == 0.0) return;
                 const double ir = rsqrt_nr(r2);
                 const double r = r2 * ir;
                 const double e[3] = {x0 * ir, x1 * ir, x2 * ir};
@@ -1187,7 +1249,7 @@ __device__ void p_cell(const DevSK &sk, const DftbArgs &a, const PbcDev &pl, SH 
                 double fc, dfc;
                 cutoff_fn(r, sk, fc, dfc);
                 g_sr = fma(rsqrt_nr(r2 + c2) - ir, fc, g_sr);
-            }
+            });
             // block (mu of A, nu of B) at column oB + nu, row oA + mu, and its transpose; a block of an
             // atom with its own images is symmetric, written as the mean of the two halves
             for (int mu = 0; mu < na; ++mu)
@@ -1747,8 +1809,9 @@ __device__ void p_cell(const DevSK &sk, const DftbArgs &a, const PbcDev &pl, SH 
             }
             __syncthreads();
             const double *W = H;
-            for (int t = j; t < nat * (nat + 1) / 2; t += PT) {   // pairs A <= B, packed by A
-                const int A = lower_col(t, nat), B = A + (t - (A * nat - A * (A - 1) / 2));
+            for (int t = j; t < nat * (nat + 1) / 2; t += PT) {   // pairs A <= B, by kind
+                int A, B;
+                pbc_pair(sh, nat, t, A, B);
                 const int eA = sh.spec[A], eB = sh.spec[B];
                 const int oA = sh.atom_off[A], oB = sh.atom_off[B];
                 const int na = sk.norb[eA], nb = sk.norb[eB];
@@ -1764,22 +1827,22 @@ __device__ void p_cell(const DevSK &sk, const DftbArgs &a, const PbcDev &pl, SH 
                 double gk[3] = {0.0, 0.0, 0.0};
                 double erep = 0.0;
                 if (A != B && first) {
-                    for (int im = 0; im < pl.n_img; ++im) {   // real-space Ewald gradient
+                    pbc_images(pl, dw, pl.n_img, pl.r_real2, [&](int im) {   // real-space Ewald gradient
                         const double x0 = dw[0] + pl.img[3 * im], x1 = dw[1] + pl.img[3 * im + 1], x2 = dw[2] + pl.img[3 * im + 2];
                         const double r2 = fma(x0, x0, fma(x1, x1, x2 * x2));
-                        if (!(r2 < pl.r_real2) || r2 == 0.0) continue;
+                        if (!(r2 < pl.r_real2) || r2 == 0.0) return;
                         const double ir = rsqrt_nr(r2);
                         const double ar = pl.alpha * (r2 * ir);
                         const double rad = -qq * (erfc(ar) * ir + two_a_spi * exp(-ar * ar)) * ir * ir;
                         gk[0] = fma(rad, x0, gk[0]);
                         gk[1] = fma(rad, x1, gk[1]);
                         gk[2] = fma(rad, x2, gk[2]);
-                    }
+                    });
                 }
-                for (int im = 0; im < pl.n_img_sk; ++im) {   // images within r_cut
+                pbc_images(pl, dw, pl.n_img_sk, rc2, [&](int im) {   // images within r_cut
                     const double x0 = dw[0] + pl.img[3 * im], x1 = dw[1] + pl.img[3 * im + 1], x2 = dw[2] + pl.img[3 * im + 2];
                     const double r2 = fma(x0, x0, fma(x1, x1, x2 * x2));
-                    if (!(r2 < rc2) || r2 == 0.0) continue;
+                    if (!(r2 < rc2) || r2 == 0.0) return;
                     const double ir = rsqrt_nr(r2);
                     const double r = r2 * ir;
                     const double e[3] = {x0 * ir, x1 * ir, x2 * ir};
@@ -1862,7 +1925,7 @@ __device__ void p_cell(const DevSK &sk, const DftbArgs &a, const PbcDev &pl, SH 
                         for (int k = 0; k < 3; ++k) gk[k] = fma(2.0, g[k], gk[k]);
                     }
                     for (int k = 0; k < 3; ++k) gk[k] = fma(rad, e[k], gk[k]);
-                }
+                });
                 double *pb = pbuf + 4LL * (A * nat + B);
                 if (fresh) {
                     pb[0] = gk[0];
@@ -1945,8 +2008,9 @@ __device__ void p_cell(const DevSK &sk, const DftbArgs &a, const PbcDev &pl, SH 
         const double *W = H;
         // pair tasks A <= B: d/dr_B of every image term (band, overlap, second order, repulsion), and
         // the repulsion energy (an atom with its own images counts each image pair once)
-        for (int t = j; t < nat * (nat + 1) / 2; t += PT) {   // pairs A <= B, packed by A
-            const int A = lower_col(t, nat), B = A + (t - (A * nat - A * (A - 1) / 2));
+        for (int t = j; t < nat * (nat + 1) / 2; t += PT) {   // pairs A <= B, by kind
+            int A, B;
+                pbc_pair(sh, nat, t, A, B);
             const int eA = sh.spec[A], eB = sh.spec[B];
             const int oA = sh.atom_off[A], oB = sh.atom_off[B];
             const int na = sk.norb[eA], nb = sk.norb[eB];
@@ -1963,22 +2027,22 @@ __device__ void p_cell(const DevSK &sk, const DftbArgs &a, const PbcDev &pl, SH 
             double gk[3] = {0.0, 0.0, 0.0};
             double erep = 0.0;
             if (A != B) {
-                for (int im = 0; im < pl.n_img; ++im) {   // real-space Ewald gradient
+                pbc_images(pl, dw, pl.n_img, pl.r_real2, [&](int im) {   // real-space Ewald gradient
                     const double x0 = dw[0] + pl.img[3 * im], x1 = dw[1] + pl.img[3 * im + 1], x2 = dw[2] + pl.img[3 * im + 2];
                     const double r2 = fma(x0, x0, fma(x1, x1, x2 * x2));
-                    if (!(r2 < pl.r_real2) || r2 == 0.0) continue;
+                    if (!(r2 < pl.r_real2) || r2 == 0.0) return;
                     const double ir = rsqrt_nr(r2);
                     const double ar = pl.alpha * (r2 * ir);
                     const double rad = -qq * (erfc(ar) * ir + two_a_spi * exp(-ar * ar)) * ir * ir;
                     gk[0] = fma(rad, x0, gk[0]);
                     gk[1] = fma(rad, x1, gk[1]);
                     gk[2] = fma(rad, x2, gk[2]);
-                }
+                });
             }
-            for (int im = 0; im < pl.n_img_sk; ++im) {   // images within r_cut
+            pbc_images(pl, dw, pl.n_img_sk, rc2, [&](int im) {   // images within r_cut
                 const double x0 = dw[0] + pl.img[3 * im], x1 = dw[1] + pl.img[3 * im + 1], x2 = dw[2] + pl.img[3 * im + 2];
                 const double r2 = fma(x0, x0, fma(x1, x1, x2 * x2));
-                if (!(r2 < rc2) || r2 == 0.0) continue;
+                if (!(r2 < rc2) || r2 == 0.0) return;
                 const double ir = rsqrt_nr(r2);
                 const double r = r2 * ir;
                 const double e[3] = {x0 * ir, x1 * ir, x2 * ir};
@@ -2047,7 +2111,7 @@ __device__ void p_cell(const DevSK &sk, const DftbArgs &a, const PbcDev &pl, SH 
                     }
                 }
                 for (int k = 0; k < 3; ++k) gk[k] = fma(rad, e[k], gk[k]);
-            }
+            });
             double *pb = pbuf + 4LL * (A * nat + B);
             pb[0] = gk[0];
             pb[1] = gk[1];
