@@ -1009,8 +1009,7 @@ __device__ __noinline__ void scc_general_water(const DftbArgs &a, MolShared<3, 6
 // Lanes: six per water, lane = orbital = matrix row. A row of S and of H0 stays in registers, so a
 // product with C needs only broadcast reads of C; products over rows go through shared memory.
 // The radial functions of a pair stay in registers for the gradient.
-__global__ void __launch_bounds__(256, 1) k_water_warm(const DevSK *__restrict__ skp, const DftbArgs a, const int gpw) {
-    const DevSK &sk = *skp;
+__device__ __forceinline__ void water_warm(const DevSK &sk, const DftbArgs &a, const int gpw) {
     using SM = MolShared<3, 6>;
     constexpr int LD = SM::LD;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1721,6 +1720,18 @@ __global__ void __launch_bounds__(256, 1) k_water_warm(const DevSK *__restrict__
     }
 }
 
+// 200 registers: eight warps per SM without spills, the faster code while that many warps hold the batch.
+__global__ void __launch_bounds__(256, 1) k_water_warm(const DevSK *__restrict__ skp, const DftbArgs a, const int gpw) {
+    water_warm(*skp, a, gpw);
+}
+
+// 128 registers (252 bytes of spills): twelve warps per SM, for batches of more than eight warps per SM.
+// Passes of 262,144 waters x 50 steps 138.5 -> 132.5 ms; of 8 waters x 30 steps 1.61 -> 1.66 ms.
+__global__ void __launch_bounds__(256, 2) k_water_warm_dense(const DevSK *__restrict__ skp, const DftbArgs a,
+                                                             const int gpw) {
+    water_warm(*skp, a, gpw);
+}
+
 __global__ void k_born_assemble(int n_cells, const int *__restrict__ off, const double *__restrict__ M0,
                                 const double *__restrict__ Md, int nd, int central, double h,
                                 double *__restrict__ b) {
@@ -1760,8 +1771,14 @@ cudaError_t launch_dftb_water(const DevSK *sk, const DftbArgs &a, cudaStream_t s
     const int blocks = (int)((rows + per_block - 1) / per_block);
     const size_t smem = sizeof(SM) * per_block;
     if (a.n_cells <= 0) return cudaSuccess;
-    if (a.have_warm && a.warm_water) k_water_warm<<<blocks, threads, smem, st>>>(sk, a, gpw);
-    else dftb_kernel<NAT, NORB><<<blocks, threads, smem, st>>>(sk, a, gpw);
+    if (a.have_warm && a.warm_water) {
+        int dev = 0, n_sm = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+        if (e != cudaSuccess) return e;
+        if ((long long)blocks * warps > 8LL * n_sm) k_water_warm_dense<<<blocks, threads, smem, st>>>(sk, a, gpw);
+        else k_water_warm<<<blocks, threads, smem, st>>>(sk, a, gpw);
+    } else dftb_kernel<NAT, NORB><<<blocks, threads, smem, st>>>(sk, a, gpw);
     return cudaGetLastError();
 }
 
@@ -1769,5 +1786,7 @@ cudaError_t prepare_dftb_water(int max_warps) {
     const int smem = (int)(sizeof(MolShared<3, 6>) * max_warps * 5);
     const cudaError_t e = cudaFuncSetAttribute(dftb_kernel<3, 6>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(k_water_warm, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    const cudaError_t e2 = cudaFuncSetAttribute(k_water_warm, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e2 != cudaSuccess) return e2;
+    return cudaFuncSetAttribute(k_water_warm_dense, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
 }

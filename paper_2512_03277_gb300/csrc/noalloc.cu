@@ -18,54 +18,72 @@
 
 namespace {
 
-constexpr int NA_CELLS = 32;
-constexpr int NA_SLICES = 32;
+constexpr int NA_THREADS = 256;
+constexpr int NA_CELLS = 32;      // cells per block for more than NA_MAX_BLOCKS x NA_CELLS_FINE cells,
+constexpr int NA_CELLS_FINE = 16; // and up to there
 constexpr int NA_MAX_BLOCKS = CAVMD_NOALLOC_MAX_CELLS / NA_CELLS;
 
 // partials [0, NA_MAX_BLOCKS), then one slot whose first word is the last-block counter
 static __device__ __align__(256) double noalloc_scratch[NA_MAX_BLOCKS + 32];
 
-__global__ void __launch_bounds__(NA_CELLS *NA_SLICES)
+// CELLS cells x 256 / CELLS mode slices per block. One FP64 multiply-add per element of U, so the FP64
+// pipe bounds it (16,384 x 1024: 27.6 us; U itself is 20 us of HBM). Blocks of 16 cells split that size
+// into 6.7 blocks per SM, all resident, where 1024-thread blocks of 32 cells ran one and two thirds
+// waves; eight loads per thread in flight hide the latency. The kick takes every thread of the block: one
+// Cartesian component of an atom each (cells own consecutive atoms, so the block's atoms are a range).
+template <int CELLS>
+__global__ void __launch_bounds__(NA_THREADS)
 k_field_kick_noalloc(int N, int M, const int *__restrict__ off, const double *__restrict__ U,
                      const double *__restrict__ W, const double *__restrict__ F,
                      const double *__restrict__ b, const double *__restrict__ inv_mass, double tau,
                      double *__restrict__ p, double *__restrict__ E_out, double *__restrict__ e_kin,
                      double *__restrict__ scratch) {
-    __shared__ double red[NA_SLICES][NA_CELLS];
+    constexpr int SLICES = NA_THREADS / CELLS, NW = NA_THREADS / 32;
+    __shared__ double red[SLICES][CELLS];
+    __shared__ double es[CELLS];
+    __shared__ int o[CELLS + 1];
+    __shared__ double part[NW];
     __shared__ bool last;
     unsigned *counter = reinterpret_cast<unsigned *>(scratch + NA_MAX_BLOCKS);
-    const int cl = threadIdx.x & (NA_CELLS - 1);
-    const int sl = threadIdx.x / NA_CELLS;
-    const int n = blockIdx.x * NA_CELLS + cl;
+    const int cl = threadIdx.x & (CELLS - 1);
+    const int sl = threadIdx.x / CELLS;
+    const int n0 = blockIdx.x * CELLS, n = n0 + cl;
+    if (threadIdx.x <= CELLS) o[threadIdx.x] = off[min(n0 + (int)threadIdx.x, N)];
     double e = 0.0;
     if (n < N) {
         const double *u = U + n;
 #pragma unroll 8
-        for (int al = sl; al < M; al += NA_SLICES) e = fma(u[(size_t)al * N], __ldg(W + al), e);
+        for (int al = sl; al < M; al += SLICES) e = fma(u[(size_t)al * N], __ldg(W + al), e);
     }
     red[sl][cl] = e;
     __syncthreads();
-    double kin = 0.0;
-    if (sl == 0 && n < N) {
-        for (int s = 1; s < NA_SLICES; ++s) e += red[s][cl];
-        if (E_out) E_out[n] = e;
-        for (int j = off[n]; j < off[n + 1]; ++j) {
-            const double im = inv_mass[j];
-            for (int k = 0; k < 3; ++k) {
-                const double pj = fma(tau, F[3 * j + k], fma(e, b[3 * j + k], p[3 * j + k]));
-                p[3 * j + k] = pj;
-                kin = fma(0.5 * im * pj, pj, kin);
-            }
-        }
-    }
     if (sl == 0) {
+        for (int s = 1; s < SLICES; ++s) e += red[s][cl];
+        es[cl] = e;
+        if (E_out && n < N) E_out[n] = e;
+    }
+    __syncthreads();
+    double kin = 0.0;
+    for (int i = 3 * o[0] + threadIdx.x; i < 3 * o[CELLS]; i += NA_THREADS) {
+        const int j = i / 3;
+        int c = 0;   // the cell of atom j: the last one that starts at or before it
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) kin += __shfl_xor_sync(CAVMD_FULL_MASK, kin, o);
-        if (cl == 0) {
-            scratch[blockIdx.x] = kin;
-            __threadfence();
-            last = (atomicAdd(counter, 1u) == gridDim.x - 1);
-        }
+        for (int h = CELLS / 2; h > 0; h >>= 1)
+            if (o[c + h] <= j) c += h;
+        const double pj = fma(tau, F[i], fma(es[c], b[i], p[i]));
+        p[i] = pj;
+        kin = fma(0.5 * inv_mass[j] * pj, pj, kin);
+    }
+#pragma unroll
+    for (int h = 16; h > 0; h >>= 1) kin += __shfl_xor_sync(CAVMD_FULL_MASK, kin, h);
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = kin;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double t = 0.0;
+        for (int w = 0; w < NW; ++w) t += part[w];
+        scratch[blockIdx.x] = t;
+        __threadfence();
+        last = (atomicAdd(counter, 1u) == gridDim.x - 1);
     }
     __syncthreads();
     if (!last) return;
@@ -73,12 +91,12 @@ k_field_kick_noalloc(int N, int M, const int *__restrict__ off, const double *__
     double v = 0.0;
     for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) v += __ldcg(scratch + i);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(CAVMD_FULL_MASK, v, o);
-    if (cl == 0) red[0][sl] = v;
+    for (int h = 16; h > 0; h >>= 1) v += __shfl_xor_sync(CAVMD_FULL_MASK, v, h);
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = v;
     __syncthreads();
     if (threadIdx.x == 0) {
         double t = 0.0;
-        for (int w = 0; w < NA_SLICES; ++w) t += red[0][w];
+        for (int w = 0; w < NW; ++w) t += part[w];
         *e_kin = t;
         *counter = 0u;
     }
@@ -145,10 +163,14 @@ extern "C" int cavmd_field_kick_noalloc(int32_t n_cells, int32_t n_modes, const 
         cavmd_set_global_error(std::string("cavmd_field_kick_noalloc: cudaMemsetAsync: ") + cudaGetErrorString(e));
         return CAVMD_ERR_CUDA;
     }
-    const int blocks = (n_cells + NA_CELLS - 1) / NA_CELLS;
-    k_field_kick_noalloc<<<blocks, NA_CELLS * NA_SLICES, 0, st>>>(
-        n_cells, n_modes, cell_offset, U, W, F, b, inv_mass, tau, p, E_out, e_kin_out,
-        static_cast<double *>(scratch));
+    if (n_cells <= NA_MAX_BLOCKS * NA_CELLS_FINE)
+        k_field_kick_noalloc<NA_CELLS_FINE><<<(n_cells + NA_CELLS_FINE - 1) / NA_CELLS_FINE, NA_THREADS, 0, st>>>(
+            n_cells, n_modes, cell_offset, U, W, F, b, inv_mass, tau, p, E_out, e_kin_out,
+            static_cast<double *>(scratch));
+    else
+        k_field_kick_noalloc<NA_CELLS><<<(n_cells + NA_CELLS - 1) / NA_CELLS, NA_THREADS, 0, st>>>(
+            n_cells, n_modes, cell_offset, U, W, F, b, inv_mass, tau, p, E_out, e_kin_out,
+            static_cast<double *>(scratch));
     e = cudaGetLastError();
     if (e != cudaSuccess) {
         cavmd_set_global_error(std::string("cavmd_field_kick_noalloc: launch: ") + cudaGetErrorString(e));
