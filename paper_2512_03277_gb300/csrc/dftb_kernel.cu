@@ -1004,8 +1004,8 @@ __device__ __noinline__ void scc_general_water(const DftbArgs &a, MolShared<3, 6
 // the FP32 part but the starting basis and the approximate Hessian enters the result. A water that
 // leaves the path's range (a rotation above W_ROT_MAX, a Hessian or gap that is not safely positive,
 // no convergence) goes through the general solve of its warp.
-// Measured (GB300, one launch): 262,144 waters 6.31 -> 2.08 ms, 4,096 waters 156 -> 48 us; mean
-// evaluations 6.15 -> 2.09. Bound: the FP64 pipe at large batches, the serial chain at small ones.
+// Measured (GB300, one launch): 262,144 waters 6.31 -> 2.0 ms, 4,096 waters 156 -> 47 us; mean
+// evaluations 6.15 -> 2.04. Bound: the FP64 pipe at large batches, the serial chain at small ones.
 // Lanes: six per water, lane = orbital = matrix row. A row of S and of H0 stays in registers, so a
 // product with C needs only broadcast reads of C; products over rows go through shared memory.
 // The radial functions of a pair stay in registers for the gradient.
@@ -1184,8 +1184,9 @@ __device__ __forceinline__ void water_warm(const DevSK &sk, const DftbArgs &a, c
 #pragma unroll
         for (int i = 0; i < 6; ++i) load_row(w.Mf[i], M[i]);
     };
-    const float u0 = (float)U0, u1 = (float)U1, u2 = (float)U2;
-    const float zf0 = (float)z0, zf1 = (float)z1, zf2 = (float)z2;
+    const float u0 = d2f_steer(U0), u1 = d2f_steer(U1), u2 = d2f_steer(U2);
+    const float zf0 = d2f_steer(z0), zf1 = d2f_steer(z1), zf2 = d2f_steer(z2);
+    const double hU0 = 0.5 * U0, hU1 = 0.5 * U1, hU2 = 0.5 * U2, h01 = 0.5 * g01, h02 = 0.5 * g02, h12 = 0.5 * g12;
     const float f01 = d2f_steer(g01), f02 = d2f_steer(g02), f12 = d2f_steer(g12);
     bool ok = true;
     {
@@ -1422,7 +1423,7 @@ __device__ __forceinline__ void water_warm(const DevSK &sk, const DftbArgs &a, c
     put_C();
 
     // ---------------------------------------------------------------- FP64 evaluations
-    double q0 = 0.0, q1 = 0.0, q2 = 0.0, s0 = 0.0, s1 = 0.0, s2 = 0.0;   // populations, half shifts
+    double q0 = 0.0, q1 = 0.0, q2 = 0.0, s0 = 0.0, s1 = 0.0, s2 = 0.0;   // populations of one spin, half shifts
     // q(C), the shifts and H C_occ (in X) of the basis in w.C
     auto evaluate = [&]() {
         double x[4] = {0.0, 0.0, 0.0, 0.0};
@@ -1435,15 +1436,15 @@ __device__ __forceinline__ void water_warm(const DevSK &sk, const DftbArgs &a, c
             x[2] = fma(sr[i], hi.x, x[2]);
             x[3] = fma(sr[i], hi.y, x[3]);
         }
-        if (act) w.pop[j] = 2.0 * fma(c[0], x[0], fma(c[1], x[1], fma(c[2], x[2], c[3] * x[3])));
+        if (act) w.pop[j] = fma(c[0], x[0], fma(c[1], x[1], fma(c[2], x[2], c[3] * x[3])));   // of one spin
         __syncwarp();
         q0 = (w.pop[0] + w.pop[1]) + (w.pop[2] + w.pop[3]);
         q1 = w.pop[4];
         q2 = w.pop[5];
-        const double d0 = 0.5 * (q0 - z0), d1 = 0.5 * (q1 - z1), d2 = 0.5 * (q2 - z2);
-        s0 = fma(U0, d0, fma(g01, d1, g02 * d2));
-        s1 = fma(g01, d0, fma(U1, d1, g12 * d2));
-        s2 = fma(g02, d0, fma(g12, d1, U2 * d2));
+        const double d0 = fma(2.0, q0, -z0), d1 = fma(2.0, q1, -z1), d2 = fma(2.0, q2, -z2);
+        s0 = fma(hU0, d0, fma(h01, d1, h02 * d2));
+        s1 = fma(h01, d0, fma(hU1, d1, h12 * d2));
+        s2 = fma(h02, d0, fma(h12, d1, hU2 * d2));
         const double sj = j < 4 ? s0 : (j == 4 ? s1 : s2);
         const double t0 = sj + s0, t1 = sj + s1, t2 = sj + s2;
         double h[6];
@@ -1486,7 +1487,7 @@ __device__ __forceinline__ void water_warm(const DevSK &sk, const DftbArgs &a, c
         float L[36], rhs[8], K[8];
 #pragma unroll
         for (int i = 0; i < 36; ++i) L[i] = w.L[i];
-        float amax = 0.0f, move = 0.0f;
+        float amax = 0.0f, move1 = 0.0f, move2 = 0.0f;
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
             rhs[i] = w.av[i];
@@ -1494,7 +1495,11 @@ __device__ __forceinline__ void water_warm(const DevSK &sk, const DftbArgs &a, c
         }
         w_solve(L, rhs, K);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) move = fmaf(4.0f * (fabsf(w.B[i]) + fabsf(w.B[8 + i])), fabsf(K[i]), move);
+        for (int i = 0; i < 8; ++i) {   // the charges' change under K (the oxygen's is minus the sum)
+            move1 = fmaf(4.0f * w.B[i], K[i], move1);
+            move2 = fmaf(4.0f * w.B[8 + i], K[i], move2);
+        }
+        const float move = fmaxf(fabsf(move1 + move2), fmaxf(fabsf(move1), fabsf(move2)));
         if (!conv && ok) {
             used = it;
             conv = amax < (float)EIG_TOL && move < tol;
@@ -1570,6 +1575,10 @@ __device__ __forceinline__ void water_warm(const DevSK &sk, const DftbArgs &a, c
         put_C();
         evaluate();
     }
+
+    q0 *= 2.0;
+    q1 *= 2.0;
+    q2 *= 2.0;
 
     if (disp) {   // finite-difference row: only the dipole of the converged charges
         if (valid && j == 0) {
@@ -1725,8 +1734,9 @@ __global__ void __launch_bounds__(256, 1) k_water_warm(const DevSK *__restrict__
     water_warm(*skp, a, gpw);
 }
 
-// 128 registers (252 bytes of spills): twelve warps per SM, for batches of more than eight warps per SM.
-// Passes of 262,144 waters x 50 steps 138.5 -> 132.5 ms; of 8 waters x 30 steps 1.61 -> 1.66 ms.
+// 128 registers with spills: twelve warps per SM, for batches of more than 24 warps per SM (two of its waves).
+// Passes of 262,144 waters x 50 steps 138.5 -> 132.5 ms; of 8 waters x 30 steps 1.61 -> 1.66 ms, and 14.6
+// warps per SM of displaced rows (1,237 waters x 9 steps) 0.92 -> 0.96 ms.
 __global__ void __launch_bounds__(256, 2) k_water_warm_dense(const DevSK *__restrict__ skp, const DftbArgs a,
                                                              const int gpw) {
     water_warm(*skp, a, gpw);
@@ -1776,7 +1786,7 @@ cudaError_t launch_dftb_water(const DevSK *sk, const DftbArgs &a, cudaStream_t s
         cudaError_t e = cudaGetDevice(&dev);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
         if (e != cudaSuccess) return e;
-        if ((long long)blocks * warps > 8LL * n_sm) k_water_warm_dense<<<blocks, threads, smem, st>>>(sk, a, gpw);
+        if ((long long)blocks * warps > 24LL * n_sm) k_water_warm_dense<<<blocks, threads, smem, st>>>(sk, a, gpw);
         else k_water_warm<<<blocks, threads, smem, st>>>(sk, a, gpw);
     } else dftb_kernel<NAT, NORB><<<blocks, threads, smem, st>>>(sk, a, gpw);
     return cudaGetLastError();
