@@ -384,12 +384,25 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) k_tc_forward(int n_stage_total
     if (warp == 0) tc::tmem_dealloc(tmem, 2 * TC);
 }
 
-__global__ void k_tc_reduce(int n_part, int size, const double *__restrict__ partial, double *__restrict__ G) {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= size) return;
+// Eight threads per entry, a contiguous eighth of the partials each, then their sums in order: a chain of
+// 19 loads instead of 152 bounds the launch (22.5 -> 7.3 us at 128 x 32 entries, one thread per entry before).
+constexpr int RED_E = 32, RED_S = 8;
+__global__ void __launch_bounds__(RED_E *RED_S) k_tc_reduce(int n_part, int size, const double *__restrict__ partial,
+                                                            double *__restrict__ G) {
+    __shared__ double red[RED_S][RED_E];
+    const int l = threadIdx.x % RED_E, sl = threadIdx.x / RED_E, e = blockIdx.x * RED_E + l;
+    const int per = (n_part + RED_S - 1) / RED_S, p1 = min(n_part, (sl + 1) * per);
     double s = 0.0;
-    for (int p = 0; p < n_part; ++p) s += partial[(size_t)p * size + e];
-    G[e] = s;
+    if (e < size) {
+#pragma unroll 4
+        for (int p = sl * per; p < p1; ++p) s += partial[(size_t)p * size + e];
+    }
+    red[sl][l] = s;
+    __syncthreads();
+    if (sl == 0 && e < size) {
+        for (int k = 1; k < RED_S; ++k) s += red[k][l];
+        G[e] = s;
+    }
 }
 
 // Back product, persistent over tiles of 128 cells: D[n][i] = sum_j Y[n][j] Wt[i][j] (cells on the
@@ -632,7 +645,7 @@ cudaError_t launch_tc_forward(const TcPlan &p, const double *Mc, double *G, unsi
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const int size = KXP * p.KY;
-    k_tc_reduce<<<(size + 255) / 256, 256, 0, st>>>(p.n_fwd_cta, size, p.partial, G);
+    k_tc_reduce<<<(size + RED_E - 1) / RED_E, RED_E * RED_S, 0, st>>>(p.n_fwd_cta, size, p.partial, G);
     return cudaGetLastError();
 }
 
