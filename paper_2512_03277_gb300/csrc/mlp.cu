@@ -486,6 +486,14 @@ __device__ __forceinline__ void load_weights_t(uint8_t *dst, const uint16_t *src
     }
 }
 
+// Eight consecutive floats at a 32-byte boundary (rows of the activations and of W3), or zeros.
+__device__ __forceinline__ void load8(const float *p, bool have, float *x) {
+    const float4 z = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    const float4 a = have ? *reinterpret_cast<const float4 *>(p) : z, b = have ? *reinterpret_cast<const float4 *>(p + 4) : z;
+    x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w;
+    x[4] = b.x; x[5] = b.y; x[6] = b.z; x[7] = b.w;
+}
+
 // Backward through the activations, per 128-atom tile on the tensor cores. With gy = dL/dy (the
 // 9 outputs, from the cell tensors):
 //   gz2[a][u] = silu'(z2[a][u]) sum_o gy[a][o] W3[o][u]      (CUDA cores, 9 terms)
@@ -494,6 +502,7 @@ __device__ __forceinline__ void load_weights_t(uint8_t *dst, const uint16_t *src
 //   gz1[a][v] = silu'(z1[a][v]) gh1[a][v]                     (TMEM epilogue)
 // gz2, gz1 and gy leave feature-major per tile ([tile][feature][atom]) for the weight gradients;
 // atoms beyond n get zeros, so they add nothing there.
+// z2, z1 and W3 are read in 32-byte pieces and z1 under the MMAs: 120 -> 66 us at 20,001 waters.
 constexpr size_t BWA_SMEM = SW2 + 3 * (size_t)A_SPLIT + ((size_t)NO * NH + MT * 16) * 4 + 64;
 
 __global__ void __launch_bounds__(FWD_THREADS, 1) k_backward_act_tc(int n, const float *__restrict__ gy,
@@ -536,18 +545,28 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) k_backward_act_tc(int n, const
             gyt[((size_t)t * 16 + o) * MT + at] = v;
         }
         __syncthreads();
+        float gy_row[NO];
+#pragma unroll
+        for (int o = 0; o < NO; ++o) gy_row[o] = gys[row * 16 + o];
 #pragma unroll
         for (int g = 0; g < 4; ++g) {
-            float x[8];
+            float x[8], z[8];
+            const int u0 = 32 * slice + 8 * g;
+            load8(z2 + (size_t)(t0 + row) * NH + u0, real, z);
+#pragma unroll
+            for (int q = 0; q < 8; ++q) x[q] = 0.0f;
+#pragma unroll
+            for (int o = 0; o < NO; ++o) {
+                float w8[8];
+                load8(w3 + o * NH + u0, true, w8);
+#pragma unroll
+                for (int q = 0; q < 8; ++q) x[q] = fmaf(gy_row[o], w8[q], x[q]);
+            }
 #pragma unroll
             for (int q = 0; q < 8; ++q) {
-                const int u = 32 * slice + 8 * g + q;
-                float acc = 0.0f;
-#pragma unroll
-                for (int o = 0; o < NO; ++o) acc = fmaf(gys[row * 16 + o], w3[o * NH + u], acc);
-                const float gz = real ? acc * dsilu(z2[(size_t)(t0 + row) * NH + u]) : 0.0f;
+                const float gz = real ? x[q] * dsilu(z[q]) : 0.0f;
                 x[q] = gz;
-                gz2t[((size_t)t * NH + u) * MT + row] = gz;
+                gz2t[((size_t)t * NH + u0 + q) * MT + row] = gz;
             }
             split_store8(sa, tc::core_offset(row, 32 * slice + 8 * g, LBO_A), x);
         }
@@ -559,6 +578,9 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) k_backward_act_tc(int n, const
             layer_mma(tmem, sa_u, sw_u, LBO_W, NH, ID128);
             tc::mma_commit(done);
         }
+        float z1r[32];   // in flight under the MMAs
+#pragma unroll
+        for (int g = 0; g < 4; ++g) load8(z1 + (size_t)(t0 + row) * NH + 32 * slice + 8 * g, real, z1r + 8 * g);
         const bool mg = tc::mbar_wait(done, pd);
         pd ^= 1u;
         if (!__syncthreads_and(mg)) { ok = false; break; }
@@ -566,9 +588,12 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) k_backward_act_tc(int n, const
         float v[32];
         tc::tmem_ld32(lanes + 32 * slice, v);
 #pragma unroll
-        for (int q = 0; q < 32; ++q) {
-            const int u = 32 * slice + q;
-            gz1t[((size_t)t * NH + u) * MT + row] = real ? v[q] * dsilu(z1[(size_t)(t0 + row) * NH + u]) : 0.0f;
+        for (int g = 0; g < 4; ++g) {
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                const int u = 32 * slice + 8 * g + q;
+                gz1t[((size_t)t * NH + u) * MT + row] = real ? v[8 * g + q] * dsilu(z1r[8 * g + q]) : 0.0f;
+            }
         }
         tc::fence_before_sync();
         __syncthreads();   // TMEM read and gy tile consumed before the next tile
@@ -596,35 +621,49 @@ constexpr uint32_t WG_OP = 2 * (3 * WGA + WGB1 + WGB2 + WGB3);
 constexpr size_t WG_SMEM = WG_OP + 64;
 constexpr uint32_t D2COL = 160, D3COL = 224;
 
-// Rows [0, R_src) of a feature-major tile (rows of MT atoms) for atoms chunk*32 .. +31, the ones row
-// (if any) and zero rows up to R, split into BF16 hi / lo in the K-major core layout (K = atoms).
-__device__ __forceinline__ void wg_operand(uint8_t *hi, uint8_t *lo, const float *src, int R_src, int ones, int R,
-                                           int chunk) {
-    const uint32_t lbo = (uint32_t)(R / 8) * 128;
-    for (int c = threadIdx.x; c < R * (WG_K / 8); c += WG_THREADS) {
-        const int g = c / R, r = c - g * R;
-        float x[8];
-        if (r < R_src) {
-            const float *p = src + (size_t)r * MT + chunk * WG_K + 8 * g;
-            const float4 u0 = *reinterpret_cast<const float4 *>(p), u1 = *reinterpret_cast<const float4 *>(p + 4);
-            x[0] = u0.x; x[1] = u0.y; x[2] = u0.z; x[3] = u0.w;
-            x[4] = u1.x; x[5] = u1.y; x[6] = u1.z; x[7] = u1.w;
-        } else {
-            const float f = r == ones ? 1.0f : 0.0f;
+// Rows [0, R_SRC) of a feature-major tile (rows of MT atoms) for atoms chunk*32 .. +31, the row of ones
+// (ONES, if any) and zero rows up to R: this thread's groups of 8 atoms, loaded into registers, and later
+// split into BF16 hi / lo in the K-major core layout (K = atoms).
+template <int R, int R_SRC, int ONES>
+struct WgOperand {
+    static constexpr int ITEMS = R * (WG_K / 8), PER = (ITEMS + WG_THREADS - 1) / WG_THREADS;
+    float4 x[PER][2];
+    __device__ __forceinline__ void load(const float *src, int chunk) {
 #pragma unroll
-            for (int q = 0; q < 8; ++q) x[q] = f;
+        for (int i = 0; i < PER; ++i) {
+            const int c = threadIdx.x + i * WG_THREADS, g = c / R, r = c - g * R;
+            if (c < ITEMS && r < R_SRC) {
+                const float *p = src + (size_t)r * MT + chunk * WG_K + 8 * g;
+                x[i][0] = *reinterpret_cast<const float4 *>(p);
+                x[i][1] = *reinterpret_cast<const float4 *>(p + 4);
+            } else {
+                const float f = r == ONES ? 1.0f : 0.0f;
+                x[i][0] = x[i][1] = make_float4(f, f, f, f);
+            }
         }
-        uint4 ph, pl;
-        ph.x = bf16x2_split(x[0], x[1]); ph.y = bf16x2_split(x[2], x[3]);
-        ph.z = bf16x2_split(x[4], x[5]); ph.w = bf16x2_split(x[6], x[7]);
-        pl.x = bf16x2_split(x[0], x[1]); pl.y = bf16x2_split(x[2], x[3]);
-        pl.z = bf16x2_split(x[4], x[5]); pl.w = bf16x2_split(x[6], x[7]);
-        const uint32_t off = tc::core_offset(r, 8 * g, lbo);
-        *reinterpret_cast<uint4 *>(hi + off) = ph;
-        *reinterpret_cast<uint4 *>(lo + off) = pl;
     }
-}
+    __device__ __forceinline__ void store(uint8_t *hi, uint8_t *lo) const {
+        constexpr uint32_t lbo = (uint32_t)(R / 8) * 128;
+#pragma unroll
+        for (int i = 0; i < PER; ++i) {
+            const int c = threadIdx.x + i * WG_THREADS, g = c / R, r = c - g * R;
+            if (c >= ITEMS) continue;
+            float v[8] = {x[i][0].x, x[i][0].y, x[i][0].z, x[i][0].w, x[i][1].x, x[i][1].y, x[i][1].z, x[i][1].w};
+            uint4 ph, pl;
+            ph.x = bf16x2_split(v[0], v[1]); ph.y = bf16x2_split(v[2], v[3]);
+            ph.z = bf16x2_split(v[4], v[5]); ph.w = bf16x2_split(v[6], v[7]);
+            pl.x = bf16x2_split(v[0], v[1]); pl.y = bf16x2_split(v[2], v[3]);
+            pl.z = bf16x2_split(v[4], v[5]); pl.w = bf16x2_split(v[6], v[7]);
+            const uint32_t off = tc::core_offset(r, 8 * g, lbo);
+            *reinterpret_cast<uint4 *>(hi + off) = ph;
+            *reinterpret_cast<uint4 *>(lo + off) = pl;
+        }
+    }
+};
 
+// The chunks of all tiles are dealt out evenly (13 at most of 1876 on 152 CTAs at 20,001 waters, where whole
+// tiles gave 16), and the next chunk's operands are loaded into registers while this chunk's MMAs run:
+// 117 -> 72 us at 20,001 waters. Bound: staging (conversion to BF16 and shared stores) and one thread's MMA issue.
 __global__ void __launch_bounds__(WG_THREADS, 1) k_weight_grad_tc(int n, const float *__restrict__ gz2t,
                                                                 const float *__restrict__ gz1t,
                                                                 const float *__restrict__ h1t,
@@ -651,22 +690,42 @@ __global__ void __launch_bounds__(WG_THREADS, 1) k_weight_grad_tc(int n, const f
     float db3 = 0.0f;   // thread o < 9: sum over this CTA's atoms of gy[.][o]
     uint32_t pd = 0u;
     bool ok = true, first = true, pending = false;
-    for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
-        if (tid < NO)
-            for (int at = 0; at < MT; ++at) db3 += gyt[((size_t)t * 16 + tid) * MT + at];
-        for (int ch = 0; ch < MT / WG_K; ++ch) {
+    WgOperand<NH, NH, -1> oa1, oa2, oa3;
+    WgOperand<WN1, NH, NH> ob1;
+    WgOperand<WN2, NF, NF> ob2;
+    WgOperand<WN3, NO, -1> ob3;
+    constexpr int CH = MT / WG_K;
+    const int n_chunks = n_tiles * CH;
+    const int c_lo = (int)((long long)blockIdx.x * n_chunks / gridDim.x), c_hi = (int)((long long)(blockIdx.x + 1) * n_chunks / gridDim.x);
+    auto load = [&](int cc) {
+        const size_t t = cc / CH;
+        const int ch = cc % CH;
+        oa1.load(gz2t + t * NH * MT, ch);
+        oa2.load(gz1t + t * NH * MT, ch);
+        oa3.load(h2t + t * NH * MT, ch);
+        ob1.load(h1t + t * NH * MT, ch);
+        ob2.load(xt + t * NF * MT, ch);
+        ob3.load(gyt + t * 16 * MT, ch);
+    };
+    if (c_lo < c_hi) load(c_lo);
+    for (int cc = c_lo; cc < c_hi && ok; ++cc) {
+        {
             if (pending) {   // the previous chunk's MMAs read the operands: wait before overwriting
                 const bool mg = tc::mbar_wait(done, pd);
                 pd ^= 1u;
                 pending = false;
                 if (!__syncthreads_and(mg)) { ok = false; break; }
             }
-            wg_operand(a1h, a1l, gz2t + (size_t)t * NH * MT, NH, -1, NH, ch);
-            wg_operand(a2h, a2l, gz1t + (size_t)t * NH * MT, NH, -1, NH, ch);
-            wg_operand(a3h, a3l, h2t + (size_t)t * NH * MT, NH, -1, NH, ch);
-            wg_operand(b1h, b1l, h1t + (size_t)t * NH * MT, NH, NH, WN1, ch);
-            wg_operand(b2h, b2l, xt + (size_t)t * NF * MT, NF, NF, WN2, ch);
-            wg_operand(b3h, b3l, gyt + (size_t)t * 16 * MT, NO, -1, WN3, ch);
+            oa1.store(a1h, a1l);
+            oa2.store(a2h, a2l);
+            oa3.store(a3h, a3l);
+            ob1.store(b1h, b1l);
+            ob2.store(b2h, b2l);
+            ob3.store(b3h, b3l);
+            if (tid < NO) {
+                const float *gp = gyt + ((size_t)(cc / CH) * 16 + tid) * MT + (cc % CH) * WG_K;
+                for (int at = 0; at < WG_K; ++at) db3 += gp[at];
+            }
             tc::fence_proxy_async();
             tc::fence_before_sync();
             __syncthreads();
@@ -699,6 +758,7 @@ __global__ void __launch_bounds__(WG_THREADS, 1) k_weight_grad_tc(int n, const f
             }
             pending = true;
             first = false;
+            if (cc + 1 < c_hi) load(cc + 1);
         }
     }
     if (pending) {
@@ -819,23 +879,40 @@ __global__ void k_cell_tensors(int n_cells, const int *__restrict__ off, const f
     }
 }
 
-__global__ void k_reduce_grad(int n_tiles, const float *__restrict__ part, float *__restrict__ g) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= NPAR) return;
+// Eight threads per parameter, a contiguous eighth of the partials each, then their sums in order.
+constexpr int RG_P = 32, RG_S = 8;
+__global__ void __launch_bounds__(RG_P *RG_S) k_reduce_grad(int n_tiles, const float *__restrict__ part,
+                                                            float *__restrict__ g) {
+    __shared__ double red[RG_S][RG_P];
+    const int l = threadIdx.x % RG_P, sl = threadIdx.x / RG_P, p = blockIdx.x * RG_P + l;
+    const int per = (n_tiles + RG_S - 1) / RG_S, t1 = min(n_tiles, (sl + 1) * per);
     double s = 0.0;
-    for (int t = 0; t < n_tiles; ++t) s += part[(size_t)t * NPAR + p];
-    g[p] = (float)s;
+    if (p < NPAR) {
+#pragma unroll 4
+        for (int t = sl * per; t < t1; ++t) s += part[(size_t)t * NPAR + p];
+    }
+    red[sl][l] = s;
+    __syncthreads();
+    if (sl == 0 && p < NPAR) {
+        for (int k = 1; k < RG_S; ++k) s += red[k][l];
+        g[p] = (float)s;
+    }
 }
 
-__global__ void k_reduce_loss(int n, const double *__restrict__ part, double scale, double *__restrict__ out) {
-    __shared__ double red[256];
+constexpr int RL_THREADS = 1024;
+__global__ void __launch_bounds__(RL_THREADS) k_reduce_loss(int n, const double *__restrict__ part, double scale,
+                                                            double *__restrict__ out) {
+    __shared__ double red[RL_THREADS / 32];
     double s = 0.0;
-    for (int i = threadIdx.x; i < n; i += 256) s += part[i];
-    red[threadIdx.x] = s;
+#pragma unroll 8
+    for (int i = threadIdx.x; i < n; i += RL_THREADS) s += part[i];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(CAVMD_FULL_MASK, s, o);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
     __syncthreads();
     if (threadIdx.x == 0) {
         double t = 0.0;
-        for (int i = 0; i < 256; ++i) t += red[i];
+        for (int i = 0; i < RL_THREADS / 32; ++i) t += red[i];
         *out = t * scale;
     }
 }
@@ -1008,8 +1085,8 @@ int mlp_loss_grad_range(cavmd_mlp *m, int cell0, int ncells, const float *X, con
                                                                   m->gyt, m->status);
     k_weight_grad_tc<<<grid, WG_THREADS, WG_SMEM, m->stream>>>(na, m->gz2t, m->gz1t, m->h1t, m->h2t, m->xt, m->gyt,
                                                                m->part, m->status);
-    k_reduce_grad<<<(NPAR + 255) / 256, 256, 0, m->stream>>>(grid, m->part, m->g);
-    k_reduce_loss<<<1, 256, 0, m->stream>>>(ncells, m->lpart, inv_count, m->loss);
+    k_reduce_grad<<<(NPAR + RG_P - 1) / RG_P, RG_P * RG_S, 0, m->stream>>>(grid, m->part, m->g);
+    k_reduce_loss<<<1, RL_THREADS, 0, m->stream>>>(ncells, m->lpart, inv_count, m->loss);
     MCK(cudaGetLastError());
     return CAVMD_OK;
 }
