@@ -980,30 +980,32 @@ int build_context(cavmd_ctx *c, const cavmd_system *sys, const cavmd_sk_tables *
     if (c->periodic) {
         PbcPlan &pp = c->pplan;
         std::vector<double> img, gw;
-        plan_dftb_periodic(sys->lattice, sk->r_cut, pp, img, gw);
+        std::vector<int4> gi;
+        pp.amax = 0;
+        for (int n = 0; n < N; ++n) pp.amax = std::max(pp.amax, sys->cell_offset[n + 1] - sys->cell_offset[n]);
+        plan_dftb_periodic(sys->lattice, sk->r_cut, pp.amax, pp, img, gw, gi);
         if (pp.n_img > 200000 || pp.n_g > 20000)
             return fail(c, CAVMD_ERR_UNSUPPORTED, "lattice too thin: " + std::to_string(pp.n_img) + " lattice images");
         pp.nmax = 0;
-        pp.amax = 0;
         pp.nk = nk;
-        for (int n = 0; n < N; ++n) {
+        for (int n = 0; n < N; ++n)
             pp.nmax = std::max(pp.nmax, (int)std::lround(std::sqrt((double)(coff[n + 1] - coff[n]) /
                                                                    (nk > 0 ? 4.0 * nk : 1.0))));
-            pp.amax = std::max(pp.amax, sys->cell_offset[n + 1] - sys->cell_offset[n]);
-        }
         int nsm = 0;
         CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device));
         CK(prepare_dftb_periodic());
         CK(plan_dftb_periodic_launch(pp, N, nsm));
         AL(pp.d_img, img.size());
         AL(pp.d_gw, gw.size());
-        AL(pp.work, pbc_workspace_doubles(pp.nmax, pp.amax, pp.n_g, nk, pp.cluster) * (size_t)pp.blocks);
+        AL(pp.d_gi, gi.size());
+        AL(pp.work, pbc_workspace_doubles(pp.nmax, pp.amax, pp.n_g, pp.g_max, nk, pp.cluster) * (size_t)pp.blocks);
         if (nk > 0) {
             AL(pp.d_kpt, kpts.size());
             CK(cudaMemcpyAsync(pp.d_kpt, kpts.data(), sizeof(double) * kpts.size(), cudaMemcpyHostToDevice, st));
         }
         CK(cudaMemcpyAsync(pp.d_img, img.data(), sizeof(double) * img.size(), cudaMemcpyHostToDevice, st));
         CK(cudaMemcpyAsync(pp.d_gw, gw.data(), sizeof(double) * gw.size(), cudaMemcpyHostToDevice, st));
+        CK(cudaMemcpyAsync(pp.d_gi, gi.data(), sizeof(int4) * gi.size(), cudaMemcpyHostToDevice, st));
         AL(c->d_Coff, N);
         CK(cudaMemcpyAsync(c->d_Coff, coff.data(), sizeof(long long) * N, cudaMemcpyHostToDevice, st));
         CK(cudaStreamSynchronize(st));   // the host vectors must outlive the copies

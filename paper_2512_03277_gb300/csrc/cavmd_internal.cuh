@@ -255,6 +255,8 @@ cudaError_t launch_dftb_generic(const DevSK *sk_dev, const DftbArgs &a, const Ge
 struct PbcPlan {
     double lat[9], inv[9];                // lattice vectors as rows; inverse (f = r inv)
     double alpha, bg, self_e, r_real;     // Ewald splitting, background and self terms, real-space cutoff
+    int n_g32, g_max;                     // reciprocal vectors that matter in FP32; largest |integer coordinate|
+    int4 *d_gi;                           // device: [n_g] integer coordinates of the reciprocal vectors
     int n_img, n_img_sk, n_g;             // lattice translations (by length; the first n_img_sk reach
                                           // r_cut); half-space reciprocal vectors
     int nmax, amax;                       // largest cell
@@ -264,12 +266,12 @@ struct PbcPlan {
     int nk;                               // k-grid: irreducible k-points (0: Gamma point only)
     double *d_kpt;                        // device: [nk][4] fractional k and weight
 };
-size_t pbc_workspace_doubles(int nmax, int amax, int n_g, int nk, int cluster);
+size_t pbc_workspace_doubles(int nmax, int amax, int n_g, int g_max, int nk, int cluster);
 const void *pbc_kg_small();   // the k-grid kernels (problems up to 256 and up to 512 wide)
 const void *pbc_kg_large();
 std::vector<double> pbc_kpoints(const int *kgrid);
-void plan_dftb_periodic(const double *lat, double r_cut, PbcPlan &p, std::vector<double> &img,
-                        std::vector<double> &gw);
+void plan_dftb_periodic(const double *lat, double r_cut, int n_atoms, PbcPlan &p, std::vector<double> &img,
+                        std::vector<double> &gw, std::vector<int4> &gi);
 cudaError_t prepare_dftb_periodic();   // kernel attributes, before plan_dftb_periodic_launch
 cudaError_t plan_dftb_periodic_launch(PbcPlan &p, int n_cells, int n_sm);
 cudaError_t launch_dftb_periodic(const DevSK *sk_dev, const DftbArgs &a, const PbcPlan &p, cudaStream_t st);

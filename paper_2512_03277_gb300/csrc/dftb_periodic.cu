@@ -25,9 +25,9 @@ __global__ void __launch_bounds__(PT, 2) k_dftb_periodic(const DevSK *__restrict
 // ---------------------------------------------------------------------------------------------
 // Host side
 
-size_t pbc_workspace_doubles(int nmax, int amax, int n_g, int nk, int cluster) {
+size_t pbc_workspace_doubles(int nmax, int amax, int n_g, int g_max, int nk, int cluster) {
     const size_t n2 = (nk > 0 ? 4 : 1) * (size_t)nmax * nmax, k = nk > 0 ? nk : 1, a2 = (size_t)amax * amax;
-    const size_t own = 6 * n2 + 2 * (size_t)n_g + 4 * a2 + (a2 + 1) / 2;
+    const size_t own = 6 * n2 + 2 * (size_t)n_g + 4 * a2 + (a2 + 1) / 2 + 6 * (size_t)amax * (g_max + 1) + 1;
     return (nk > 0 ? 5 : 3) * k * n2 + a2 + 2 * (size_t)amax * n_g + 2 * (size_t)cluster * (amax + 8) + cluster * own + 32;
 }
 
@@ -53,10 +53,12 @@ std::vector<double> pbc_kpoints(const int *kgrid) {
 }
 
 // Lattice images and reciprocal vectors for one lattice (rows a_i), and the Ewald constants. The
-// splitting parameter is chosen so the half-space reciprocal list holds about 1000 vectors; every
-// term left out of either sum is below 1e-18 (erfc(6.5) and exp(-6.5^2)).
-void plan_dftb_periodic(const double *lat, double r_cut, PbcPlan &p, std::vector<double> &img,
-                        std::vector<double> &gw) {
+// splitting parameter is chosen so the half-space reciprocal list holds about 250 sqrt(n_atoms) vectors, at
+// least 1000: the real-space sums cost n_atoms^2 / n_g error functions, the reciprocal ones n_atoms n_g
+// products (99 atoms: 22 images a pair at 1000 vectors, 9 at 2500). Every term left out of either sum is
+// below 1e-18 (erfc(6.5) and exp(-6.5^2)).
+void plan_dftb_periodic(const double *lat, double r_cut, int n_atoms, PbcPlan &p, std::vector<double> &img,
+                        std::vector<double> &gw, std::vector<int4> &gi) {
     for (int k = 0; k < 9; ++k) p.lat[k] = lat[k];
     const double a0 = lat[0], a1 = lat[1], a2 = lat[2], b0 = lat[3], b1 = lat[4], b2 = lat[5], c0 = lat[6],
                  c1 = lat[7], c2 = lat[8];
@@ -70,8 +72,8 @@ void plan_dftb_periodic(const double *lat, double r_cut, PbcPlan &p, std::vector
     const double V = std::fabs(det);
     const double EX = 6.5;
     const double pi = 3.141592653589793;
-    // half-space count N ~ (4 pi / 3) (2 alpha EX)^3 V / (2 (2 pi)^3)  ->  alpha for N = 1000
-    const double g_cube = 1000.0 * 2.0 * std::pow(2.0 * pi, 3) * 3.0 / (4.0 * pi * V);
+    // half-space count N ~ (4 pi / 3) (2 alpha EX)^3 V / (2 (2 pi)^3)  ->  alpha for N
+    const double g_cube = std::max(1000.0, 250.0 * std::sqrt((double)n_atoms)) * 2.0 * std::pow(2.0 * pi, 3) * 3.0 / (4.0 * pi * V);
     const double alpha = std::cbrt(g_cube) / (2.0 * EX);
     p.alpha = alpha;
     p.bg = -pi / (alpha * alpha * V);
@@ -123,7 +125,8 @@ void plan_dftb_periodic(const double *lat, double r_cut, PbcPlan &p, std::vector
         const double an = std::sqrt(lat[3 * i] * lat[3 * i] + lat[3 * i + 1] * lat[3 * i + 1] + lat[3 * i + 2] * lat[3 * i + 2]);
         M[i] = (int)std::ceil(g_max * an / (2.0 * pi)) + 1;
     }
-    gw.clear();
+    struct Vec { double g2, G[3], w2; int m[3]; };
+    std::vector<Vec> vs;
     for (int m0 = -M[0]; m0 <= M[0]; ++m0)
         for (int m1 = -M[1]; m1 <= M[1]; ++m1)
             for (int m2 = -M[2]; m2 <= M[2]; ++m2) {
@@ -134,11 +137,19 @@ void plan_dftb_periodic(const double *lat, double r_cut, PbcPlan &p, std::vector
                 const double g2 = G[0] * G[0] + G[1] * G[1] + G[2] * G[2];
                 if (!(g2 < g_max * g_max)) continue;
                 const double w = 4.0 * pi / V * std::exp(-g2 / (4.0 * alpha * alpha)) / g2;
-                gw.push_back(G[0]);
-                gw.push_back(G[1]);
-                gw.push_back(G[2]);
-                gw.push_back(2.0 * w);
+                vs.push_back({g2, {G[0], G[1], G[2]}, 2.0 * w, {m0, m1, m2}});
             }
+    std::stable_sort(vs.begin(), vs.end(), [](const Vec &x, const Vec &y) { return x.g2 < y.g2; });
+    gw.clear();
+    gi.clear();
+    p.n_g32 = 0;
+    p.g_max = 0;
+    for (const Vec &v : vs) {
+        gw.insert(gw.end(), {v.G[0], v.G[1], v.G[2], v.w2});
+        gi.push_back(make_int4(v.m[0], v.m[1], v.m[2], 0));
+        if (v.g2 < 4.0 * alpha * alpha * 18.0) ++p.n_g32;   // exp(-18) = 1.5e-8 of the weight at small G
+        for (int k = 0; k < 3; ++k) p.g_max = std::max(p.g_max, std::abs(v.m[k]));
+    }
     p.n_g = (int)(gw.size() / 4);
 }
 
@@ -215,12 +226,15 @@ cudaError_t launch_dftb_periodic(const DevSK *sk_dev, const DftbArgs &a, const P
     d.n_img = p.n_img;
     d.n_img_sk = p.n_img_sk;
     d.n_g = p.n_g;
+    d.n_g32 = p.n_g32;
+    d.g_max = p.g_max;
+    d.gi = p.d_gi;
     d.nmax = p.nmax;
     d.amax = p.amax;
     d.img = p.d_img;
     d.gw = p.d_gw;
     d.work = p.work;
-    d.work_stride = (long long)pbc_workspace_doubles(p.nmax, p.amax, p.n_g, p.nk, p.cluster);
+    d.work_stride = (long long)pbc_workspace_doubles(p.nmax, p.amax, p.n_g, p.g_max, p.nk, p.cluster);
     d.nk = p.nk;
     d.cluster = p.cluster;
     d.kpt = p.d_kpt;

@@ -274,6 +274,8 @@ struct PbcDev {
     double alpha, bg, self_e;    // Ewald alpha, -pi / (alpha^2 V), -2 alpha / sqrt(pi)
     double r_real2;              // real-space cutoff squared
     int n_img, n_img_sk, n_g, nmax, amax;
+    int n_g32, g_max;            // vectors that matter in FP32; largest |m| of a vector
+    const int4 *gi;              // [n_g] the vectors' integer coordinates
     const double *img;           // [n_img][3] lattice translations by increasing length; the first
                                  // n_img_sk reach every image within r_cut
     const double *gw;            // [n_g][4] half-space reciprocal vectors G and 2 w_G
@@ -295,6 +297,7 @@ struct PbcMem {
     double *H0, *S;                     // Gamma: the matrices; k-grid: of the first k-point, 2 n2 apart
     float *kf;                          // k-grid: FP32 state of every k-point, 4 n2 floats apart
     double *gam, *csg;                  // real-space gamma; cos and sin of G . r
+    double *pw;                         // this block's powers of the reciprocal phases
     double *Cd;                         // bases of a finite-difference copy
     double *xch;                        // [2][blocks][amax + 8] exchange between the blocks of a cell
 };
@@ -397,15 +400,23 @@ __device__ __noinline__ void p_shifts(SH &sh, const PbcDev &pl, const PbcMem &w,
         w.sgf[2 * g + 1] = ss;
     }
     __syncthreads();
+    // every thread: atom j % nat, a contiguous share of the vectors; the shares are added in order
+    const int parts = PT / nat, part = j / nat, at = j - part * nat, per = (pl.n_g + parts - 1) / parts;
+    if (part < parts) {
+        const int g1 = min(pl.n_g, (part + 1) * per);
+        double rr = 0.0;
+        for (int g = part * per; g < g1; ++g) {
+            const double *t = w.csg + 2LL * (g * nat + at);
+            rr = fma(pl.gw[4 * g + 3], fma(t[0], w.sgf[2 * g], t[1] * w.sgf[2 * g + 1]), rr);
+        }
+        sh.Xs[j] = rr;
+    }
+    __syncthreads();
     if (j < nat) {
         double v = 0.0;
         for (int k = 0; k < nat; ++k) v = fma(w.gam[j * pl.amax + k], sh.dq[k], v);
-        double rr = 0.0;
-        for (int g = 0; g < pl.n_g; ++g) {
-            const double *t = w.csg + 2LL * (g * nat + j);
-            rr = fma(pl.gw[4 * g + 3], fma(t[0], w.sgf[2 * g], t[1] * w.sgf[2 * g + 1]), rr);
-        }
-        sh.shift[j] = v + rr;
+        for (int q = 0; q < parts; ++q) v += sh.Xs[q * nat + j];
+        sh.shift[j] = v;
     }
     __syncthreads();
 }
@@ -637,13 +648,23 @@ __device__ __noinline__ bool p_warm(const DftbArgs &a, const PbcDev &pl, SH &sh,
     };
 
     // ---------------------------------------------------------------- gamma in FP32
-    fprod<5, 5, false, false>(sh, nat, nat, 2 * pl.n_g,
-                              [&](int A, int k) { return d2f_steer(wk.csg[2LL * ((long long)(k >> 1) * nat + A) + (k & 1)]); },
-                              [&](int k, int B) {
-                                  return d2f_steer(pl.gw[4 * (k >> 1) + 3]) *
-                                         d2f_steer(wk.csg[2LL * ((long long)(k >> 1) * nat + B) + (k & 1)]);
-                              },
-                              [&](int A, int B, float v) { wk.g32[B * nat + A] = v + d2f_steer(wk.gam[A * pl.amax + B]); });
+    // The vectors are sorted by length: from n_g32 on their weights are below FP32 rounding of gamma. Slices of
+    // 32 vectors are added in FP64 (in pbuf): a single FP32 sum over them all was 5e-7 off, enough for the
+    // Hessian to ask for a third evaluation.
+    for (int e = j; e < nat * nat; e += PT) wk.pbuf[e] = wk.gam[(e % nat) * pl.amax + e / nat];
+    __syncthreads();
+    for (int g0 = 0; g0 < pl.n_g32; g0 += 32) {
+        const int k0 = 2 * g0;
+        fprod<7, 7, false, false>(sh, nat, nat, 2 * min(32, pl.n_g32 - g0),
+                                  [&](int A, int k) { return d2f_steer(wk.csg[2LL * ((long long)((k0 + k) >> 1) * nat + A) + (k & 1)]); },
+                                  [&](int k, int B) {
+                                      return d2f_steer(pl.gw[4 * ((k0 + k) >> 1) + 3]) *
+                                             d2f_steer(wk.csg[2LL * ((long long)((k0 + k) >> 1) * nat + B) + (k & 1)]);
+                                  },
+                                  [&](int A, int B, float v) { wk.pbuf[B * nat + A] += f2d_steer(v); });
+    }
+    for (int e = j; e < nat * nat; e += PT) wk.g32[e] = __double2float_rn(wk.pbuf[e]);
+    __syncthreads();
 
     // ---------------------------------------------------------------- FP32 start
     float big = 0.0f;
@@ -877,9 +898,9 @@ __device__ __noinline__ bool p_warm(const DftbArgs &a, const PbcDev &pl, SH &sh,
                         pd = pd && d > 0.0f;
                         const int end = k < mo ? mo : m;
                         const float id = 1.0f / d;
-                        for (int c = k + 1 + j; c < end; c += PT) {   // column c of the trailing block (symmetric storage)
+                        for (int c = k + 1 + (j >> 5); c < end; c += PT / 32) {   // a warp per column of the trailing block
                             const float f = A32[k * m + c] * id;
-                            for (int i = c; i < end; ++i) A32[c * m + i] = fmaf(-f, A32[k * m + i], A32[c * m + i]);
+                            for (int i = c + (j & 31); i < end; i += 32) A32[c * m + i] = fmaf(-f, A32[k * m + i], A32[c * m + i]);
                         }
                         __syncthreads();
                     }
@@ -889,7 +910,7 @@ __device__ __noinline__ bool p_warm(const DftbArgs &a, const PbcDev &pl, SH &sh,
                 return true;
             }
         }
-        if (it == most || !newton(1e-6f)) return false;
+        if (it == most || !newton(1e-7f)) return false;   // (1e-6 left one cell in ten above scc_tol)
         float kmax = 0.0f;
         for (int kp = rank; kp < NKP; kp += blocks) {
             set_k(kp);
@@ -1269,16 +1290,38 @@ __device__ void p_cell(const DevSK &sk, const DftbArgs &a, const PbcDev &pl, SH 
             gam[B * pl.amax + A] = gv;
         }
     }
-    // cos and sin of G . (r_A - r_0) for the reciprocal sum
-    for (int e = j + rank * PT; e < nat * pl.n_g; e += blocks * PT) {
-        const int g = e / nat, at = e - g * nat;
-        const double *G = pl.gw + 4 * g;
-        const double ph = fma(G[0], sh.pos[at][0] - sh.pos[0][0],
-                              fma(G[1], sh.pos[at][1] - sh.pos[0][1], G[2] * (sh.pos[at][2] - sh.pos[0][2])));
-        double sn, cn;
-        sincos(ph, &sn, &cn);
-        csg[2LL * e] = cn;
-        csg[2LL * e + 1] = sn;
+    // cos and sin of G . (r_A - r_0) for the reciprocal sum:
+    // G = m0 b0 + m1 b1 + m2 b2: products of three powers of exp(i b . (r_A - r_0)), so a (vector, atom) takes
+    // two complex products instead of a sincos. The powers: [axis][0..g_max][atom].
+    {
+        double2 *pw = reinterpret_cast<double2 *>(wk.pw);
+        const int gm = pl.g_max + 1;
+        for (int e = j; e < 3 * nat; e += PT) {
+            const int ax = e / nat, at = e - ax * nat;
+            const double turns = fma(sh.pos[at][0] - sh.pos[0][0], pl.inv[ax],
+                                     fma(sh.pos[at][1] - sh.pos[0][1], pl.inv[3 + ax], (sh.pos[at][2] - sh.pos[0][2]) * pl.inv[6 + ax]));
+            double sn, cn;
+            sincospi(2.0 * turns, &sn, &cn);
+            double x = 1.0, y = 0.0;
+            for (int q = 0; q < gm; ++q) {
+                pw[(ax * gm + q) * nat + at] = make_double2(x, y);
+                const double u = fma(x, cn, -y * sn);
+                y = fma(x, sn, y * cn);
+                x = u;
+            }
+        }
+        __syncthreads();
+        for (int e = j + rank * PT; e < nat * pl.n_g; e += blocks * PT) {
+            const int g = e / nat, at = e - g * nat;
+            const int4 q = pl.gi[g];   // m0 >= 0 or the vector is the half space's; signs by conjugation
+            double2 a0 = pw[abs(q.x) * nat + at], a1 = pw[(gm + abs(q.y)) * nat + at], a2 = pw[(2 * gm + abs(q.z)) * nat + at];
+            a0.y = q.x < 0 ? -a0.y : a0.y;
+            a1.y = q.y < 0 ? -a1.y : a1.y;
+            a2.y = q.z < 0 ? -a2.y : a2.y;
+            const double u = fma(a0.x, a1.x, -a0.y * a1.y), v = fma(a0.x, a1.y, a0.y * a1.x);
+            csg[2LL * e] = fma(u, a2.x, -v * a2.y);
+            csg[2LL * e + 1] = fma(u, a2.y, v * a2.x);
+        }
     }
     cluster_barrier(blocks);
 
@@ -2124,14 +2167,27 @@ __device__ void p_cell(const DevSK &sk, const DftbArgs &a, const PbcDev &pl, SH 
         cluster_barrier(blocks);
         return;
     }
-    if (j < nat) {
-        // reciprocal part: d/dr_A of 1/2 sum_G w_G |S(G)|^2 = dq_A sum_G w_G G (c_A S_s - s_A S_c)
-        double gr[3] = {0.0, 0.0, 0.0};
-        for (int g = 0; g < pl.n_g; ++g) {
-            const double *t = csg + 2LL * (g * nat + j);
-            const double amp = pl.gw[4 * g + 3] * fma(t[0], sgf[2 * g + 1], -t[1] * sgf[2 * g]);
-            for (int k = 0; k < 3; ++k) gr[k] = fma(amp, pl.gw[4 * g + k], gr[k]);
+    // reciprocal part: d/dr_A of 1/2 sum_G w_G |S(G)|^2 = dq_A sum_G w_G G (c_A S_s - s_A S_c), the vectors in
+    // contiguous shares as in p_shifts
+    const int gparts = PT / nat;
+    {
+        const int part = j / nat, at = j - part * nat, per = (pl.n_g + gparts - 1) / gparts;
+        if (part < gparts) {
+            const int g1 = min(pl.n_g, (part + 1) * per);
+            double gr[3] = {0.0, 0.0, 0.0};
+            for (int g = part * per; g < g1; ++g) {
+                const double *t = csg + 2LL * (g * nat + at);
+                const double amp = pl.gw[4 * g + 3] * fma(t[0], sgf[2 * g + 1], -t[1] * sgf[2 * g]);
+                for (int k = 0; k < 3; ++k) gr[k] = fma(amp, pl.gw[4 * g + k], gr[k]);
+            }
+            for (int k = 0; k < 3; ++k) sh.Xs[3 * j + k] = gr[k];
         }
+        __syncthreads();
+    }
+    if (j < nat) {
+        double gr[3] = {0.0, 0.0, 0.0};
+        for (int q = 0; q < gparts; ++q)
+            for (int k = 0; k < 3; ++k) gr[k] += sh.Xs[3 * (q * nat + j) + k];
         double G[3];
         for (int k = 0; k < 3; ++k) G[k] = sh.dq[j] * gr[k];
         for (int A = 0; A < nat; ++A) {
@@ -2198,13 +2254,14 @@ __device__ __forceinline__ PbcMem pbc_mem(const PbcDev &pl, bool kg, long long g
     w.csg = p; p += 2LL * pl.amax * pl.n_g;
     w.Cd = p; p += nk * n2;
     w.xch = p; p += 2LL * blocks * (pl.amax + 8);
-    const long long own = 6 * n2 + 2LL * pl.n_g + 4 * a2 + (a2 + 1) / 2;
+    const long long own = 6 * n2 + 2LL * pl.n_g + 4 * a2 + (a2 + 1) / 2 + 6LL * pl.amax * (pl.g_max + 1) + 1;
     p += rank * own;
     w.H = p; w.Y = p + n2; w.P = p + 2 * n2; w.Xg = p + 3 * n2; w.Mo = p + 4 * n2; w.Mv = p + 5 * n2;
     p += 6 * n2;
     w.sgf = p; p += 2LL * pl.n_g;
     w.pbuf = p; p += 4 * a2;
-    w.g32 = (float *)p;
+    w.g32 = (float *)p; p += (a2 + 1) / 2;
+    w.pw = p + ((size_t)p & 8 ? 1 : 0);   // pairs of doubles
     w.pbuf_stride = own;
     return w;
 }
