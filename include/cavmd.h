@@ -247,7 +247,9 @@ typedef struct {
     double *q_pop;              /* [n_atoms] Mulliken populations                         */
     double *E_cell;             /* [n_cells] E_DFTB of every cell                         */
     double *M;                  /* [n_cells] projected dipoles                            */
-    int32_t *scc_iters;         /* [n_cells] SCC iterations of the last evaluation        */
+    int32_t *scc_iters;         /* [n_cells] SCC iterations of the last evaluation: with a
+                                   warm start, the FP64 evaluations of charges and residual
+                                   that follow the single-precision start             */
 } cavmd_eval;
 
 /* Opaque context: one propagated system on one GPU. */

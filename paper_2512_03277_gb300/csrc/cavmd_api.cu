@@ -639,7 +639,7 @@ int validate(const cavmd_system *sys, const cavmd_sk_tables *sk, const cavmd_mod
         GenericPlan gp{};
         std::vector<int2> it, dit;
         plan_dftb_generic(sys->cell_offset, sys->species, norb_e.data(), sys->n_cells, 0, gp, it, dit);
-        if (gp.smem > 227 * 1024 - 256)   // the opt-in limit per block, less the kernel's static bytes
+        if (gp.smem > GENERIC_SMEM_MAX)
             return fail(c, CAVMD_ERR_UNSUPPORTED, "cells too large for on-chip storage (" +
                         std::to_string(gp.smem) + " bytes of shared memory per block)");
     }

@@ -234,6 +234,8 @@ cudaError_t prepare_dftb_water(int max_warps);   // shared-memory attribute for 
 cudaError_t launch_trial_positions(const double *r, const double *p, const double *inv_mass, double dt, int n_atoms,
                                    double *r_trial, cudaStream_t st);
 
+constexpr size_t GENERIC_SMEM_MAX = 227 * 1024 - 256;   // the opt-in limit per block, less the kernel's static bytes
+
 // Plan of the persistent SCC-DFTB launch over cells of any composition (up to 64 orbitals).
 struct GenericPlan {
     int nmax_b, amax_b, nmax_s, amax_s;          // largest cell of the large (> 32 orbitals) and small classes
@@ -241,6 +243,7 @@ struct GenericPlan {
     int n_sm, blocks_per_sm, max_blocks_per_sm;  // persistent grid: n_sm x blocks_per_sm blocks
     int r_entries;                               // product entries per thread per pass (2 or 4)
     size_t smem;                                 // dynamic shared memory per block
+    int warm;                                    // the layout holds the warm path's buffer
     int2 *items, *disp_items;                    // device: (cell, -1) and (cell, displacement), largest first
     unsigned *queue;                             // device: [2] work counters
 };

@@ -14,9 +14,9 @@ cudaError_t set_attr(const void *kernel, size_t smem, int &blocks_per_sm) {
 
 }  // namespace
 
-size_t dftb_generic_smem(int nmax_b, int amax_b, int nmax_s, int amax_s) {
-    const size_t b = nmax_b > 0 ? g_layout(nmax_b, amax_b).total : 0;
-    const size_t s = nmax_s > 0 ? 2 * (size_t)g_layout(nmax_s, amax_s).total : 0;
+size_t dftb_generic_smem(int nmax_b, int amax_b, int nmax_s, int amax_s, int warm) {
+    const size_t b = nmax_b > 0 ? g_layout(nmax_b, amax_b, warm).total : 0;
+    const size_t s = nmax_s > 0 ? 2 * (size_t)g_layout(nmax_s, amax_s, warm).total : 0;
     return std::max(b, s);
 }
 
@@ -46,7 +46,13 @@ void plan_dftb_generic(const int *cell_offset, const int *species, const int *no
         items.push_back(make_int2(c, -1));
         for (int k = 0; k < n_disp_per_atom * nat; ++k) disp_items.push_back(make_int2(c, k));
     }
-    p.smem = dftb_generic_smem(p.nmax_b, p.amax_b, p.nmax_s, p.amax_s);
+    // cells of 64 orbitals with more than about 45 atoms leave no room for the warm path's buffer
+    p.warm = 1;
+    p.smem = dftb_generic_smem(p.nmax_b, p.amax_b, p.nmax_s, p.amax_s, 1);
+    if (p.smem > GENERIC_SMEM_MAX) {
+        p.warm = 0;
+        p.smem = dftb_generic_smem(p.nmax_b, p.amax_b, p.nmax_s, p.amax_s, 0);
+    }
     p.r_entries = 4;
     p.blocks_per_sm = 0;
 }
@@ -75,7 +81,9 @@ cudaError_t launch_dftb_generic(const DevSK *sk, const DftbArgs &a, const Generi
     if (e != cudaSuccess) return e;
     const int grid = std::min(units, p.n_sm * std::max(p.blocks_per_sm, 1));
     const void *kernel = p.r_entries == 2 ? dftb_generic_kernel_r2() : (const void *)k_dftb_generic<4>;
-    int nmax_b = p.nmax_b, amax_b = p.amax_b, nmax_s = p.nmax_s, amax_s = p.amax_s, n_big = nb, n_small = ns;
-    void *args[] = {(void *)&sk, (void *)&a, (void *)&items, &n_big, &n_small, &queue, &nmax_b, &amax_b, &nmax_s, &amax_s};
+    int nmax_b = p.nmax_b, amax_b = p.amax_b, nmax_s = p.nmax_s, amax_s = p.amax_s, n_big = nb, n_small = ns,
+        warm = p.warm;
+    void *args[] = {(void *)&sk, (void *)&a, (void *)&items, &n_big, &n_small, &queue, &nmax_b, &amax_b, &nmax_s, &amax_s,
+                    &warm};
     return cudaLaunchKernel(kernel, dim3(grid), dim3(BT), args, p.smem, st);
 }

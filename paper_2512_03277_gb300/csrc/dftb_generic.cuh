@@ -46,7 +46,7 @@ constexpr int TS = 128;                // threads per small cell (two per block)
 
 // Shared-memory layout of one cell (byte offsets) for cells of at most nmax orbitals, amax atoms.
 struct GLayout {
-    int nmax, amax, pmax;
+    int nmax, amax, pmax, xb;   // xb: doubles of XB (0: no warm path)
     unsigned SH, C, A, Y, Kc, XB, pos, gam, zv, q, qout, qst, shift, shl, hq, hf, red, diag, cs, invd, th, ints,
         total;
 };
@@ -55,8 +55,9 @@ struct GLayout {
 // clusters need two thirds; cells with more occupied orbitals take the general path).
 __host__ __device__ inline int g_xb(int nmax) { return (3 * nmax + 3) / 4 * (nmax + 1); }
 
-__host__ __device__ inline GLayout g_layout(int nmax, int amax) {
+__host__ __device__ inline GLayout g_layout(int nmax, int amax, int warm) {
     GLayout L;
+    L.xb = warm ? g_xb(nmax) : 0;
     L.nmax = nmax;
     L.amax = amax;
     L.pmax = amax * (amax - 1) / 2 > 0 ? amax * (amax - 1) / 2 : 1;
@@ -69,7 +70,7 @@ __host__ __device__ inline GLayout g_layout(int nmax, int amax) {
     L.A = o; o += mat;
     L.Y = o; o += ymat;
     L.Kc = o; o += (unsigned)((nmax / 2) * ((nmax + 1) / 2) + 8) * 8;   // n_occ x n_virt <= n^2 / 4
-    L.XB = o; o += (unsigned)g_xb(nmax) * 8;
+    L.XB = o; o += (unsigned)L.xb * 8;
     L.pos = o; o += amax * 3 * 8;
     L.gam = o; o += amax * amax * 8;
     L.zv = o; o += amax * 8;
@@ -867,7 +868,7 @@ __device__ void g_molecule(const DevSK &sk, const DftbArgs &a, const GLayout &L,
     const double *cw = a.Cwarm + coff;
     // ---------------------------------------------------------------- warm path
     bool warm = false;
-    if (a.have_warm && nocc > 0 && nv > 0 && nocc * LD <= g_xb(L.nmax)) {
+    if (a.have_warm && nocc > 0 && nv > 0 && nocc * LD <= L.xb) {
         GWarm wv;
         wv.n = n; wv.nocc = nocc; wv.nat = nat; wv.AM = AM;
         wv.SH = SH; wv.A = A; wv.XB = (double *)(sm + L.XB); wv.Kc = Kc; wv.gam = gam; wv.zv = zv; wv.q = q;
@@ -1454,13 +1455,13 @@ template <int R>
 __global__ void __launch_bounds__(BT, 2) k_dftb_generic(const DevSK *__restrict__ skp, const DftbArgs a,
                                                      const int2 *__restrict__ items, int n_big, int n_small,
                                                      unsigned *__restrict__ queue, int nmax_b, int amax_b,
-                                                     int nmax_s, int amax_s) {
+                                                     int nmax_s, int amax_s, int warm) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int next;
     __shared__ int vote[2][TS / 32];
     const DevSK &sk = *skp;
-    const GLayout Lb = g_layout(nmax_b, amax_b);
-    const GLayout Ls = g_layout(nmax_s, amax_s);
+    const GLayout Lb = g_layout(nmax_b, amax_b, warm);
+    const GLayout Ls = g_layout(nmax_s, amax_s, warm);
     const int n_units = n_big + (n_small + 1) / 2;
     const int half = threadIdx.x / TS;
     for (;;) {

@@ -202,7 +202,11 @@ cudaError_t plan_dftb_periodic_launch(PbcPlan &p, int n_cells, int n_sm) {
             p.blocks = std::max(1, std::min(n_cells, n));
         }
     }
-    return best < 0 ? cudaErrorInvalidConfiguration : cudaSuccess;
+    if (best < 0) return cudaErrorInvalidConfiguration;
+    // dense grids of large cells: at most 128 GiB of workspace, the blocks taking several cells in turn
+    const size_t each = 8 * pbc_workspace_doubles(p.nmax, p.amax, p.n_g, p.g_max, p.nk, p.cluster);
+    p.blocks = (int)std::max<size_t>(1, std::min<size_t>(p.blocks, ((size_t)128 << 30) / each));
+    return cudaSuccess;
 }
 
 cudaError_t prepare_dftb_periodic() {

@@ -1992,7 +1992,7 @@ __device__ void p_cell(const DevSK &sk, const DftbArgs &a, const PbcDev &pl, SH 
             double eb = 0.0;
             for (int t = 0; t < PT; ++t) eb += sh.cs[t];
             sh.red[0] = eb;
-            if (parts > 1) wk.xch[(long long)rank * (pl.amax + 8)] = eb;
+            if (rank > 0) sgf[0] = eb;   // (the structure factors are rank 0's to read from here on)
         }
         if (parts > 1) {   // rank 0 adds the others' gradients and band energies, in rank order
             cluster_barrier(blocks);
@@ -2003,7 +2003,7 @@ __device__ void p_cell(const DevSK &sk, const DftbArgs &a, const PbcDev &pl, SH 
                         for (int b = 1; b < min(parts, NKP); ++b)
                             for (int k = 0; k < 3; ++k) pbuf[4LL * e + k] += __ldcg(pbuf + b * apart + 4LL * e + k);
                 if (j == 0)
-                    for (int b = 1; b < parts; ++b) sh.red[0] += __ldcg(wk.xch + (long long)b * (pl.amax + 8));
+                    for (int b = 1; b < parts; ++b) sh.red[0] += __ldcg(sgf + b * apart);
             }
         }
         for (int r = j; r < n; r += PT)
