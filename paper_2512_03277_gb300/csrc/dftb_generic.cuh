@@ -39,6 +39,8 @@ constexpr float GW_ROT_MAX = 0.3f;     // the largest rotation taken (beyond: th
 constexpr int GW_EVALS = 8;            // and bound on the FP64 evaluations
 constexpr float GW_ORTH_MAX = 1e-4f;   // overlap defect that the second-order correction takes
 constexpr float GW_GAP = 2e-3f;        // HOMO-LUMO gap (Hartree) the warm path needs, above G_MIN_GAP
+constexpr int GW_CG_SLOW = 6;          // conjugate-gradient steps of the first Newton step that ask for a block sweep
+constexpr int GW_BISECT = 6;           // tries for a level between the occupied and the empty ones
 constexpr int GW_CG_ITERS = 40;        // bound on the conjugate-gradient steps of a Newton step
 constexpr int BT = 256;                // threads per block
 constexpr int TB = 256;                // threads per large cell
@@ -247,6 +249,8 @@ struct GWarm {
     double *SH, *A, *XB, *Kc, *gam, *zv, *q, *shift, *red;
     float *u, *dq, *ea, *eo, *scr;   // [n], [nat], [nat], [n], [8]: FP32 charges, shifts, reduction scratch
     const int *orb_atom, *atom_off;
+    int *pp, *pq;                    // pairs and
+    float *cs;                       // rotations of a Jacobi round
 };
 
 // Warm-started cell: the method of k_water_warm (dftb_kernel.cu) for matrices of any size.
@@ -387,9 +391,11 @@ __device__ bool g_warm(const DftbArgs &a, const GWarm &v, double *&C, double *&Y
     };
     // K (in x) from the residual r (destroyed): Hessian K = r to a relative residual rel, by
     // preconditioned conjugate gradients. False when the Hessian is not positive along the way.
+    int steps = 0;   // conjugate-gradient steps of the last solve
     auto newton = [&](float rel) -> bool {
         float *p = F3, *hp = F3 + nvo;
         float rz = 0.0f;
+        steps = 0;
         for (int e = j; e < nvo; e += T) {
             const float z = r[e] / diag_of(e);
             x[e] = 0.0f;
@@ -400,6 +406,7 @@ __device__ bool g_warm(const DftbArgs &a, const GWarm &v, double *&C, double *&Y
         const float stop = rel * rel * rz;
         if (!(rz < 1e30f) || !(rz >= 0.0f)) return false;
         for (int it = 0; it < GW_CG_ITERS && rz > stop; ++it) {
+            ++steps;
             charges(p);
             half_shifts();
             ftile<T, 2, 2>(j, nv, no, nv, F2 + no * LF + no, LF, 1, p, no, 1,
@@ -491,6 +498,7 @@ __device__ bool g_warm(const DftbArgs &a, const GWarm &v, double *&C, double *&Y
         g.sync();
     }
     bool done = false;
+    int first_steps = 0;
     for (int it = 0; it < GW_FP32_ITERS && !done; ++it) {
         if (it > 0) s32();
         sc32();
@@ -514,6 +522,7 @@ __device__ bool g_warm(const DftbArgs &a, const GWarm &v, double *&C, double *&Y
         }
         g.sync();
         if (!newton(it < 2 ? 3e-3f : 1e-2f)) return false;
+        if (it == 0) first_steps = steps;
         float kmax = 0.0f;
         for (int e = j; e < nvo; e += T) kmax = fmaxf(kmax, fabsf(x[e]));
         if (!all(kmax < GW_ROT_MAX)) return false;
@@ -524,6 +533,61 @@ __device__ bool g_warm(const DftbArgs &a, const GWarm &v, double *&C, double *&Y
         g.sync();
     }
     if (!done) return false;
+    // One Jacobi sweep inside each block when their off-diagonal part has grown enough to slow the solve
+    // (see p_warm in dftb_periodic.cuh); any orthogonal mixing inside a block leaves the result alone.
+    if (first_steps >= GW_CG_SLOW) {
+        for (int b = 0; b < 2; ++b) {
+            const int off = b ? no : 0, mb = b ? nv : no, me = mb + (mb & 1), half = me / 2;
+            for (int e = j; e < mb * mb; e += T) {
+                const int c = e / mb, i = e - c * mb;
+                F3[e] = F2[(off + i) * LF + off + c];
+                F4[e] = i == c ? 1.0f : 0.0f;
+            }
+            g.sync();
+            for (int rd = 0; rd < me - 1; ++rd) {
+                if (j < half) {
+                    int pa, pb;
+                    g_pair(j, rd, me, pa, pb);
+                    float t = 0.0f;
+                    if (pb < mb) {
+                        const float d = F3[pb * mb + pb] - F3[pa * mb + pa], o = 2.0f * F3[pb * mb + pa];
+                        if (o != 0.0f) t = o / (d + copysignf(sqrtf(fmaf(d, d, o * o)), d));
+                    }
+                    const float c = rsqrtf(fmaf(t, t, 1.0f));
+                    v.pp[j] = pa;
+                    v.pq[j] = pb;
+                    v.cs[2 * j] = c;
+                    v.cs[2 * j + 1] = t * c;
+                }
+                g.sync();
+                for (int e = j; e < half * 2 * mb; e += T) {   // columns of the block and of the rotation
+                    const int k = e / (2 * mb), rr = e - k * 2 * mb, pa = v.pp[k], pb = v.pq[k];
+                    if (pb >= mb) continue;
+                    float *base = rr < mb ? F3 : F4;
+                    const int i = rr < mb ? rr : rr - mb;
+                    const float xp = base[pa * mb + i], xq = base[pb * mb + i], c = v.cs[2 * k], sn = v.cs[2 * k + 1];
+                    base[pa * mb + i] = fmaf(c, xp, -sn * xq);
+                    base[pb * mb + i] = fmaf(sn, xp, c * xq);
+                }
+                g.sync();
+                for (int e = j; e < half * mb; e += T) {   // rows of the block
+                    const int k = e / mb, cc = e - k * mb, pa = v.pp[k], pb = v.pq[k];
+                    if (pb >= mb) continue;
+                    const float xp = F3[cc * mb + pa], xq = F3[cc * mb + pb], c = v.cs[2 * k], sn = v.cs[2 * k + 1];
+                    F3[cc * mb + pa] = fmaf(c, xp, -sn * xq);
+                    F3[cc * mb + pb] = fmaf(sn, xp, c * xq);
+                }
+                g.sync();
+            }
+            ftile<T, 3, 3>(j, n, mb, mb, F0 + off, LF, 1, F4, 1, mb, [&](int i, int c, float t) { F5[i * LF + c] = t; });
+            g.sync();
+            for (int e = j; e < n * mb; e += T) {
+                const int i = e / mb, c = e - i * mb;
+                F0[i * LF + off + c] = F5[i * LF + c];
+            }
+            g.sync();
+        }
+    }
 
     // ---------------------------------------------------------------- FP64: orthonormal basis
     for (int e = j; e < nn; e += T) {
@@ -634,27 +698,32 @@ __device__ bool g_warm(const DftbArgs &a, const GWarm &v, double *&C, double *&Y
                 float hi = -1e30f, lo = 1e30f;
                 for (int o = 0; o < no; ++o) hi = fmaxf(hi, F2[o * LF + o]);
                 for (int k = no; k < n; ++k) lo = fminf(lo, F2[k * LF + k]);
-                const float tau = 0.5f * (hi + lo);
-                g.sync();
-                for (int e = j; e < nn; e += T) {
-                    const int i = e / n, c = e - i * n;
-                    if (i < no && c < no) F2[i * LF + c] = (i == c ? tau : 0.0f) - F2[i * LF + c];
-                    else if (i == c) F2[i * LF + c] -= tau + GW_GAP;
-                }
-                g.sync();
-                bool pd = true;
-                for (int k = 0; k < n; ++k) {   // both blocks in turn; entries between them are not touched
-                    const float d = F2[k * LF + k];
-                    pd = pd && d > 0.0f;
-                    const int end = k < no ? no : n;
-                    const float id = 1.0f / d;
-                    for (int i = k + 1 + j; i < end; i += T) {
-                        const float f = F2[i * LF + k] * id;
-                        for (int c = k + 1; c <= i; ++c) F2[i * LF + c] = fmaf(-f, F2[c * LF + k], F2[i * LF + c]);
+                // the diagonals bound tau (mixing inside the blocks moves the levels beyond them): bisection
+                for (int t = 0;; ++t) {
+                    const float tau = 0.5f * (hi + lo);
+                    g.sync();
+                    for (int e = j; e < nn; e += T) {
+                        const int i = e / n, c = e - i * n;
+                        const float x = F2[i * LF + c];
+                        F3[i * LF + c] = (i < no && c < no) ? (i == c ? tau : 0.0f) - x : x - (i == c ? tau + GW_GAP : 0.0f);
                     }
                     g.sync();
+                    bool occ = true, emp = true;
+                    for (int k = 0; k < n; ++k) {   // both blocks in turn; entries between them are not touched
+                        const float d = F3[k * LF + k];
+                        if (k < no) occ = occ && d > 0.0f; else emp = emp && d > 0.0f;
+                        const int end = k < no ? no : n;
+                        const float id = 1.0f / d;
+                        for (int i = k + 1 + j; i < end; i += T) {
+                            const float f = F3[i * LF + k] * id;
+                            for (int c = k + 1; c <= i; ++c) F3[i * LF + c] = fmaf(-f, F3[c * LF + k], F3[i * LF + c]);
+                        }
+                        g.sync();
+                    }
+                    if (occ && emp) break;   // the same in every thread
+                    if (t == GW_BISECT || occ == emp) return false;
+                    if (occ) lo = tau; else hi = tau;
                 }
-                if (!all(pd)) return false;
                 evals = it;
                 return true;
             }
@@ -875,6 +944,7 @@ __device__ void g_molecule(const DevSK &sk, const DftbArgs &a, const GLayout &L,
         wv.shift = shift; wv.red = red;
         wv.u = (float *)diag; wv.dq = (float *)qout; wv.ea = (float *)shl; wv.eo = (float *)invd; wv.scr = (float *)th;
         wv.orb_atom = orb_atom; wv.atom_off = atom_off;
+        wv.pp = pp; wv.pq = pq; wv.cs = (float *)cs;
         g.sync();
         int evals = 0;
         warm = g_warm<T>(a, wv, C, Y, cw, g, evals);

@@ -58,6 +58,8 @@ constexpr float PW_ROT_MAX = 0.3f;      // the largest rotation taken (beyond: t
 constexpr int PW_EVALS = 8;             // and bound on the FP64 evaluations
 constexpr float PW_ORTH_MAX = 1e-4f;    // overlap defect that the second-order correction takes
 constexpr float PW_GAP = 2e-3f;         // HOMO-LUMO gap (Hartree) the warm path needs, above P_MIN_GAP
+constexpr int PW_CG_SLOW = 6;           // conjugate-gradient steps of the first Newton step that ask for a block sweep
+constexpr int PW_BISECT = 6;            // tries for a level between the occupied and the empty ones
 constexpr int PW_CG_ITERS = 60;         // bound on the conjugate-gradient steps of a Newton step
 
 // Shared memory of one block; PN is the largest problem dimension (the orbitals of a cell at the
@@ -571,8 +573,10 @@ __device__ __noinline__ bool p_warm(const DftbArgs &a, const PbcDev &pl, SH &sh,
     };
     auto diag_of = [&](int e) -> float { return A32[(mo + e % mv) * (m + 1)] - A32[(e / mv) * (m + 1)]; };
     // Hessian K = r (K in x, r destroyed) to a relative residual rel; false when it is not positive
+    int steps = 0;   // conjugate-gradient steps of the last solve
     auto newton = [&](float rel) -> bool {
         float rz = 0.0f;
+        steps = 0;
         for (int kp = rank; kp < NKP; kp += blocks) {
             set_k(kp);
             for (int e = j; e < mvo; e += PT) {
@@ -586,6 +590,7 @@ __device__ __noinline__ bool p_warm(const DftbArgs &a, const PbcDev &pl, SH &sh,
         const float stop = rel * rel * rz;
         if (!(rz < 1e30f) || !(rz >= 0.0f)) return false;
         for (int it = 0; it < PW_CG_ITERS && rz > stop; ++it) {
+            ++steps;
             charges(1);
             half_shifts();
             float ph = 0.0f;
@@ -696,6 +701,7 @@ __device__ __noinline__ bool p_warm(const DftbArgs &a, const PbcDev &pl, SH &sh,
     }
     if (!all(big < 0.2f)) return false;
     bool done = false;
+    int first_steps = 0;
     for (int it = 0; it < PW_FP32_ITERS && !done; ++it) {
         clear_u();
         for (int kp = rank; kp < NKP; kp += blocks) {
@@ -724,6 +730,7 @@ __device__ __noinline__ bool p_warm(const DftbArgs &a, const PbcDev &pl, SH &sh,
             __syncthreads();
         }
         if (!newton(it < 2 ? 3e-3f : 1e-2f)) return false;
+        if (it == 0) first_steps = steps;
         float kmax = 0.0f;
         for (int kp = rank; kp < NKP; kp += blocks) {
             set_k(kp);
@@ -740,6 +747,65 @@ __device__ __noinline__ bool p_warm(const DftbArgs &a, const PbcDev &pl, SH &sh,
         done = all(kmax < PW_FP32_KTOL);
     }
     if (!done) return false;
+    // The rotations leave the occupied and the virtual blocks of C^T H C alone, and their off-diagonal part
+    // grows with every step until the diagonal preconditioner is a poor one (100 cells of 17 waters: 11 ms a
+    // step at first, 19 after 100 steps). When the solve shows it, one Jacobi sweep inside each block (FP32:
+    // any orthogonal mixing inside a block leaves the result alone, and C is made orthonormal below).
+    if (first_steps >= PW_CG_SLOW) {
+        float *cs = (float *)sh.cs;
+        for (int kp = rank; kp < NKP; kp += blocks) {
+            set_k(kp);
+            for (int b = 0; b < 2; ++b) {
+                const int off = b ? mo : 0, mb = b ? mv : mo, me = mb + (mb & 1), half = me / 2;
+                for (int e = j; e < mb * mb; e += PT) {
+                    const int c = e / mb, i = e - c * mb;
+                    T0[e] = A32[(off + c) * m + off + i];
+                    T1[e] = i == c ? 1.0f : 0.0f;
+                }
+                __syncthreads();
+                for (int rd = 0; rd < me - 1; ++rd) {
+                    if (j < half) {
+                        int pa, pb;
+                        p_pair(j, rd, me, pa, pb);
+                        float t = 0.0f;
+                        if (pb < mb) {
+                            const float d = T0[pb * mb + pb] - T0[pa * mb + pa], o = 2.0f * T0[pb * mb + pa];
+                            if (o != 0.0f) t = o / (d + copysignf(sqrtf(fmaf(d, d, o * o)), d));
+                        }
+                        const float c = rsqrtf(fmaf(t, t, 1.0f));
+                        sh.pp[j] = pa;
+                        sh.pq[j] = pb;
+                        cs[2 * j] = c;
+                        cs[2 * j + 1] = t * c;
+                    }
+                    __syncthreads();
+                    for (int e = j; e < half * 2 * mb; e += PT) {   // columns of the block and of the rotation
+                        const int k = e / (2 * mb), rr = e - k * 2 * mb, pa = sh.pp[k], pb = sh.pq[k];
+                        if (pb >= mb) continue;
+                        float *base = rr < mb ? T0 : T1;
+                        const int i = rr < mb ? rr : rr - mb;
+                        const float xp = base[pa * mb + i], xq = base[pb * mb + i], c = cs[2 * k], sn = cs[2 * k + 1];
+                        base[pa * mb + i] = fmaf(c, xp, -sn * xq);
+                        base[pb * mb + i] = fmaf(sn, xp, c * xq);
+                    }
+                    __syncthreads();
+                    for (int e = j; e < half * mb; e += PT) {   // rows of the block
+                        const int k = e / mb, cc = e - k * mb, pa = sh.pp[k], pb = sh.pq[k];
+                        if (pb >= mb) continue;
+                        const float xp = T0[cc * mb + pa], xq = T0[cc * mb + pb], c = cs[2 * k], sn = cs[2 * k + 1];
+                        T0[cc * mb + pa] = fmaf(c, xp, -sn * xq);
+                        T0[cc * mb + pb] = fmaf(sn, xp, c * xq);
+                    }
+                    __syncthreads();
+                }
+                fprod<5, 5, false, true>(sh, m, mb, mb, [&](int i, int k) { return C32[(off + k) * m + i]; },
+                                         [&](int k, int c) { return T1[c * mb + k]; },
+                                         [&](int i, int c, float v) { SC[c * m + i] = v; });
+                for (int e = j; e < m * mb; e += PT) C32[off * m + e] = SC[e];
+                __syncthreads();
+            }
+        }
+    }
 
     // ---------------------------------------------------------------- FP64: orthonormal bases
     big = 0.0f;
@@ -872,40 +938,46 @@ __device__ __noinline__ bool p_warm(const DftbArgs &a, const PbcDev &pl, SH &sh,
                     }
                     parity ^= 1;
                 }
-                const float tau = 0.5f * (hi + lo);
-                bool pd = true;
-                for (int kp = rank; kp < NKP; kp += blocks) {
-                    set_k(kp);
-                    // a row bound first: diagonally dominant rows are enough
-                    bool dom = true;
-                    for (int i = j; i < m; i += PT) {
-                        float off = 0.0f;
-                        const int b0 = i < mo ? 0 : mo, b1 = i < mo ? mo : m;
-                        for (int c = b0; c < b1; ++c)
-                            if (c != i) off += fabsf(A32[c * m + i]);
-                        const float d = i < mo ? tau - A32[i * (m + 1)] : A32[i * (m + 1)] - tau - PW_GAP;
-                        dom = dom && d > off;
-                    }
-                    if (blk_all(dom)) continue;
-                    for (int e = j; e < mm; e += PT) {
-                        const int c = e / m, i = e - c * m;
-                        if (i < mo && c < mo) A32[e] = (i == c ? tau : 0.0f) - A32[e];
-                        else if (i == c) A32[e] -= tau + PW_GAP;
-                    }
-                    __syncthreads();
-                    for (int k = 0; k < m; ++k) {
-                        const float d = A32[k * (m + 1)];
-                        pd = pd && d > 0.0f;
-                        const int end = k < mo ? mo : m;
-                        const float id = 1.0f / d;
-                        for (int c = k + 1 + (j >> 5); c < end; c += PT / 32) {   // a warp per column of the trailing block
-                            const float f = A32[k * m + c] * id;
-                            for (int i = c + (j & 31); i < end; i += 32) A32[c * m + i] = fmaf(-f, A32[k * m + i], A32[c * m + i]);
+                // the diagonals bound tau (mixing inside the blocks moves the levels beyond them): bisection
+                for (int t = 0;; ++t) {
+                    const float tau = 0.5f * (hi + lo);
+                    bool occ = true, emp = true;
+                    for (int kp = rank; kp < NKP; kp += blocks) {
+                        set_k(kp);
+                        // a row bound first: diagonally dominant rows are enough
+                        bool dom = true;
+                        for (int i = j; i < m; i += PT) {
+                            float off = 0.0f;
+                            const int b0 = i < mo ? 0 : mo, b1 = i < mo ? mo : m;
+                            for (int c = b0; c < b1; ++c)
+                                if (c != i) off += fabsf(A32[c * m + i]);
+                            const float d = i < mo ? tau - A32[i * (m + 1)] : A32[i * (m + 1)] - tau - PW_GAP;
+                            dom = dom && d > off;
+                        }
+                        if (blk_all(dom)) continue;
+                        for (int e = j; e < mm; e += PT) {
+                            const int c = e / m, i = e - c * m;
+                            T0[e] = (i < mo && c < mo) ? (i == c ? tau : 0.0f) - A32[e] : A32[e] - (i == c ? tau + PW_GAP : 0.0f);
                         }
                         __syncthreads();
+                        for (int k = 0; k < m; ++k) {
+                            const float d = T0[k * (m + 1)];
+                            if (k < mo) occ = occ && d > 0.0f; else emp = emp && d > 0.0f;
+                            const int end = k < mo ? mo : m;
+                            const float id = 1.0f / d;
+                            for (int c = k + 1 + (j >> 5); c < end; c += PT / 32) {   // a warp per column of the trailing block
+                                const float f = T0[k * m + c] * id;
+                                for (int i = c + (j & 31); i < end; i += 32) T0[c * m + i] = fmaf(-f, T0[k * m + i], T0[c * m + i]);
+                            }
+                            __syncthreads();
+                        }
                     }
+                    occ = all(occ);
+                    emp = all(emp);
+                    if (occ && emp) break;
+                    if (t == PW_BISECT || occ == emp) return false;
+                    if (occ) lo = tau; else hi = tau;
                 }
-                if (!all(pd)) return false;
                 evals = it;
                 return true;
             }
