@@ -300,7 +300,7 @@ struct PbcMem {
     float *kf;                          // k-grid: FP32 state of every k-point, 4 n2 floats apart
     double *gam, *csg;                  // real-space gamma; cos and sin of G . r
     double *pw;                         // this block's powers of the reciprocal phases
-    double *Cd;                         // bases of a finite-difference copy
+    double *Cd;                         // working bases of the warm path and of finite-difference copies
     double *xch;                        // [2][blocks][amax + 8] exchange between the blocks of a cell
 };
 
@@ -435,15 +435,15 @@ __device__ __noinline__ void p_shifts(SH &sh, const PbcDev &pl, const PbcMem &w,
 // by C (1 + K + K^2/2) with K from the FP32 Hessian of this basis; converged when every |A_vo| < P_EIG_TOL
 // and the populations that A_vo implies to first order, q_out - q, are below scc_tol: two evaluations as a
 // rule. Nothing of the FP32 part but the starting basis and the approximate Hessian enters the result.
-// Returns false (in every block of the cell) when the cell leaves the path's range; C is then not defined
-// and the caller restores it. On success: C occupied columns first, sh.q, sh.dq and sh.shift, and for the
-// Gamma point Y = H C_o.
+// The stored bases Cs are only read; the path works in Cb (wk.Cd). Returns false (in every block of the cell)
+// when the cell leaves the path's range, so that the general path starts from Cs. On success: Cb occupied
+// columns first (each block its own k-points), sh.q, sh.dq and sh.shift, and for the Gamma point Y = H C_o.
 // Measured (GB300, one step): 304 cells of 33 waters 263 -> 76 ms (with the image lists and the Ewald split),
 // 24 cells of 8 waters on 3 x 3 x 3 232 -> 18.8 ms (with clusters of blocks); evaluations 11.8 -> 2.0. Bound: FP64
 // products (7.5 n^3 multiply-adds a cell) and pair sums, the pipe about 65 % busy.
 template <bool KG, class SH>
-__device__ __noinline__ bool p_warm(const DftbArgs &a, const PbcDev &pl, SH &sh, const PbcMem &wk, double *Cb, int n,
-                                    int nocc, int nat, int rank, int blocks, int &evals) {
+__device__ __noinline__ bool p_warm(const DftbArgs &a, const PbcDev &pl, SH &sh, const PbcMem &wk, const double *Cs,
+                                    double *Cb, int n, int nocc, int nat, int rank, int blocks, int &evals) {
     const int j = threadIdx.x;
     const int m = KG ? 2 * n : n, mo = KG ? 2 * nocc : nocc, mv = m - mo, mm = m * m, mvo = mv * mo;
     const long long n2 = (KG ? 4LL : 1LL) * pl.nmax * pl.nmax;
@@ -678,7 +678,8 @@ __device__ __noinline__ bool p_warm(const DftbArgs &a, const PbcDev &pl, SH &sh,
     float big = 0.0f;
     for (int kp = rank; kp < NKP; kp += blocks) {
         set_k(kp);
-        for (int e = j; e < mm; e += PT) C32[e] = d2f_steer(C[e]);
+        const double *from = Cs + (KG ? (long long)kp * mm : 0);
+        for (int e = j; e < mm; e += PT) C32[e] = d2f_steer(from[e]);
         __syncthreads();
         for (int pass = 0; pass < 2; ++pass) {
             build_sc();
@@ -990,6 +991,10 @@ __device__ __noinline__ bool p_warm(const DftbArgs &a, const PbcDev &pl, SH &sh,
         for (int kp = rank; kp < NKP; kp += blocks) {
             set_k(kp);
             for (int e = j; e < mvo; e += PT) kmax = fmaxf(kmax, fabsf(x[e]));
+        }
+        if (!all(kmax < 1e-2f)) return false;
+        for (int kp = rank; kp < NKP; kp += blocks) {
+            set_k(kp);
             // C (1 + K + K^2/2), as C_o + (C_v - (C_o K^T)/2) K and C_v - (C_o + (C_v K)/2) K^T; the half terms in FP32
             second(false);
             for (int e = j; e < mm; e += PT) H[e] = C[e] + f2d_steer(T1[e]);
@@ -1001,7 +1006,6 @@ __device__ __noinline__ bool p_warm(const DftbArgs &a, const PbcDev &pl, SH &sh,
                                        [&](int k, int c) { return f2d_steer(x[k * mv + c]); },
                                        [&](int i, int c, double v) { C[(long long)(mo + c) * m + i] -= v; });
         }
-        if (!all(kmax < 1e-2f)) return false;
     }
     return false;
 }
@@ -1128,12 +1132,6 @@ __device__ void p_cell(const DevSK &sk, const DftbArgs &a, const PbcDev &pl, SH 
     // the problem: orbitals (Gamma), or the real form of a k-point problem (KG)
     const int m = KG ? 2 * n : n, mo = KG ? 2 * nocc : nocc, mv = m - mo, mm = m * m;
     double *Cb = C0;   // the bases of the k-points, mm apart
-    if (disp) {   // a private copy of the cell's basis: the cell and its other copies read the original
-        for (long long e = j + (long long)rank * PT; e < (long long)NKP * mm; e += (long long)blocks * PT) wk.Cd[e] = C0[e];
-        Cb = wk.Cd;
-        C = Cb;
-        __syncthreads();
-    }
     // point the problem's matrices at k-point kp
     auto set_k = [&](int kp) {
         if (KG) {
@@ -1404,7 +1402,7 @@ __device__ void p_cell(const DevSK &sk, const DftbArgs &a, const PbcDev &pl, SH 
     bool warm = false;
     int evals = 0;
     if (a.have_warm && mo > 0 && m > mo) {
-        warm = p_warm<KG>(a, pl, sh, wk, Cb, n, nocc, nat, rank, blocks, evals);
+        warm = p_warm<KG>(a, pl, sh, wk, C0, wk.Cd, n, nocc, nat, rank, blocks, evals);
         if (j < nat) sh.qst[j] = a.qpop[a0 + j];
         if (j == 0) sh.fl[2] = evals;
         __syncthreads();
@@ -1413,6 +1411,17 @@ __device__ void p_cell(const DevSK &sk, const DftbArgs &a, const PbcDev &pl, SH 
         cluster_barrier(blocks);
         return;
     }
+    if (warm) {
+        Cb = wk.Cd;
+        if (!disp)
+            for (int kp = rank; kp < NKP; kp += blocks)
+                for (long long e = j; e < mm; e += PT) C0[(long long)kp * mm + e] = Cb[(long long)kp * mm + e];
+    } else if (disp) {   // a private copy of the cell's basis: the cell and its other copies read the original
+        for (long long e = j; e < (long long)NKP * mm; e += PT) wk.Cd[e] = C0[e];
+        Cb = wk.Cd;
+        __syncthreads();
+    }
+    C = Cb;
     // atomic shifts eps_A = sum_B gamma_AB dq_B + reciprocal part, from sh.dq
     auto shifts = [&]() { p_shifts(sh, pl, wk, nat); };
     auto build_h = [&]() {

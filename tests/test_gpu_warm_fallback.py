@@ -1,0 +1,68 @@
+"""Cells that leave the warm-started path, beside others that stay on it, against the oracles at the context's own positions. Tolerances: those of the parity tests
+(forces 1e-9 of the largest, populations and cell energies 1e-10)."""
+import numpy as np
+import pytest
+
+import cavmd_synth as cs
+from oracle import periodic as PR
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def P():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    import paper_2512_03277_gb300 as P
+    P.load_library()
+    return P
+
+
+def _check(ctx, sy, solve):
+    ev, st = ctx.cavmd_get_eval(), ctx.cavmd_get_state()
+    cells = [slice(sy.cell_offset[c], sy.cell_offset[c + 1]) for c in range(sy.n_cells)]
+    refs = [solve(sy.species[s], st["r"][s]) for s in cells]
+    largest = max(np.abs(ref["F"]).max() for ref in refs)
+    for c, (s, ref) in enumerate(zip(cells, refs)):
+        assert np.abs(ev["F_dftb"][s] - ref["F"]).max() < 1e-9 * largest
+        assert np.abs(ev["q_pop"][s] - ref["q"]).max() < 1e-10
+        assert abs(ev["E_cell"][c] - ref["E"]) < 1e-10 * max(1.0, abs(ref["E"]))
+    return ev["scc_iters"]
+
+
+def _periodic(waters, n, seed=17):
+    rng = np.random.default_rng(seed)
+    side = (waters / 33.0) ** (1.0 / 3.0) * 10.0 * cs.ANGSTROM if waters > 2 else 8.5
+    cent = np.zeros((n, 3))
+    cent[:, 0] = 200.0 * np.arange(1, n + 1)
+    kw = {} if waters > 2 else {"d_min": 4.0, "d_atom": 2.8}
+    sy, lat = cs.periodic_water_cells(rng, cent, n_waters=waters, side=side, **kw)
+    sy.p = cs.mb_momenta(rng, sy)
+    return sy, lat
+
+
+def _solver(pa, lat, grid):
+    if tuple(grid) == (1, 1, 1):
+        return lambda sp, r: PR.dftb_periodic(pa, sp, r, lat)
+    return lambda sp, r: PR.dftb_periodic_k(pa, sp, r, lat, tuple(grid))
+
+
+# the Gamma point; two points (blocks of a cluster: one or two); fourteen points (several blocks a cell, of which
+# the first takes the cell over)
+@pytest.mark.parametrize("grid", [(1, 1, 1), (2, 1, 1), (3, 3, 3)])
+def test_periodic_cells_that_leave_the_warm_path(P, grid):
+    """Every second cell's momenta four times and the time step twice as large: the overlap of those
+    cells changes by more than the warm path takes."""
+    sy, lat = _periodic(2, 4)
+    sy.p *= np.repeat(np.where(np.arange(4) % 2 == 0, 4.0, 1.0), np.diff(sy.cell_offset))[:, None]
+    o = P.default_options()
+    o.dt *= 2.0
+    o.kgrid[:] = grid
+    pa = cs.load_water_params()
+    ctx = P.Context(sy, pa, cs.line_modes(8, 1000.0, 0.001, k_max=0.01), o, lattice=lat)
+    for step in range(2):
+        ctx.cavmd_step(1)
+        it = _check(ctx, sy, _solver(pa, lat, grid))
+        if step == 0:
+            assert it.max() > 4 > it.min()   # both ways were taken
