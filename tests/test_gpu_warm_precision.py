@@ -1,0 +1,34 @@
+"""The warm-started paths leave nothing of the residual that passed their convergence test in the
+charges: against the oracle converged to 2e-14, at the context's own positions.
+
+Tolerance: scc_tol (1e-12) bounds the change that is left when the test passes, and the paths take that
+change themselves, to a tenth: 1e-13, and half of it again for the rounding of both sides and the
+oracle's own residual. (A general iteration ends likewise: it moves the basis after its test.)"""
+import numpy as np
+import pytest
+
+import cavmd_synth as cs
+from oracle import dftb as OD
+
+pytestmark = pytest.mark.gpu
+
+TOL = 1.5e-13
+
+
+@pytest.fixture(scope="module")
+def P():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    import paper_2512_03277_gb300 as P
+    P.load_library()
+    return P
+
+
+def test_waters(P):
+    w = cs.make_workload("c2", n_cells=3000, n_modes=16)
+    ctx = P.Context(w["system"], w["params"], w["modes"])
+    ctx.cavmd_step(4)
+    ev, st = ctx.cavmd_get_eval(), ctx.cavmd_get_state()
+    ref = OD.dftb(w["params"], [0, 1, 1], st["r"].reshape(-1, 3, 3), tol=2e-14, forces=False)
+    assert np.abs(ev["q_pop"].reshape(-1, 3) - ref["q"]).max() < TOL
