@@ -32,3 +32,18 @@ def test_waters(P):
     ev, st = ctx.cavmd_get_eval(), ctx.cavmd_get_state()
     ref = OD.dftb(w["params"], [0, 1, 1], st["r"].reshape(-1, 3, 3), tol=2e-14, forces=False)
     assert np.abs(ev["q_pop"].reshape(-1, 3) - ref["q"]).max() < TOL
+
+
+def test_clusters(P):
+    rng = np.random.default_rng(5)
+    sizes = list(rng.integers(1, 11, size=96))
+    sy = cs.cluster_batch(rng, sizes, np.zeros((len(sizes), 3)))
+    sy.p = cs.mb_momenta(rng, sy)
+    pa = cs.load_water_params()
+    ctx = P.Context(sy, pa, cs.line_modes(8, 1000.0, 0.001, k_max=0.01))
+    ctx.cavmd_step(4)
+    ev, st = ctx.cavmd_get_eval(), ctx.cavmd_get_state()
+    for c in range(sy.n_cells):
+        s = slice(sy.cell_offset[c], sy.cell_offset[c + 1])
+        ref = OD.dftb(pa, sy.species[s], st["r"][None, s], tol=2e-14, forces=False)
+        assert np.abs(ev["q_pop"][s] - ref["q"][0]).max() < TOL
