@@ -60,6 +60,7 @@ constexpr float PW_ORTH_MAX = 1e-4f;    // overlap defect that the second-order 
 constexpr float PW_GAP = 2e-3f;         // HOMO-LUMO gap (Hartree) the warm path needs, above P_MIN_GAP
 constexpr int PW_CG_SLOW = 6;           // conjugate-gradient steps of the first Newton step that ask for a block sweep
 constexpr int PW_BISECT = 6;            // tries for a level between the occupied and the empty ones
+constexpr float PW_LAST_TOL = 0.1f;     // relative residual of the last solve, of a rotation below 1e-9
 constexpr int PW_CG_ITERS = 60;         // bound on the conjugate-gradient steps of a Newton step
 
 // Shared memory of one block; PN is the largest problem dimension (the orbitals of a cell at the
@@ -423,6 +424,64 @@ __device__ __noinline__ void p_shifts(SH &sh, const PbcDev &pl, const PbcMem &w,
     __syncthreads();
 }
 
+// FP32 state of a k-point in the warm path: C, S C, C^T H C and K.
+struct PState32 {
+    float *C, *SC, *A, *x;
+};
+
+template <bool KG>
+__device__ __forceinline__ PState32 p_state32(const PbcMem &wk, int kp, long long n2, int mm) {
+    PState32 f;
+    f.C = KG ? wk.kf + 4LL * kp * n2 : (float *)wk.P;
+    f.SC = f.C + mm;
+    f.A = KG ? f.C + 2 * mm : (float *)wk.Xg;
+    f.x = f.A + mm;
+    return f;
+}
+
+// The end of the warm path: the residual that passed its test stays in no result. With the rotation K that it
+// asks for, q takes its change (moved), the shifts follow and C_o becomes C_o + C_v K. At the Gamma point half of
+// the change C_o^T dH C_o of A_oo goes to Mv (a k-grid forms H anew). K is solved for, to a tenth: r / (A_vv - A_oo)
+// in its place would leave half of the residual, since the blocks of A are not diagonal. Against 64 bits, 24 cells
+// of 33 waters: forces 4.2e-14 -> 5.6e-15, charges 5.2e-13 -> 2.8e-14 (without this step -> with it). A call of its own,
+// so that its registers are not p_warm's (inlined: 6,488 bytes of spill loads there instead of 3,772). 304 such cells: 73.5 -> 76.1 ms.
+template <bool KG, class SH>
+__device__ __noinline__ void p_settle(const DftbArgs &a, const PbcDev &pl, SH &sh, const PbcMem &wk, double *Cb,
+                                      const float *moved, int n, int nocc, int nat, int rank, int blocks) {
+    const int j = threadIdx.x;
+    const int m = KG ? 2 * n : n, mo = KG ? 2 * nocc : nocc, mv = m - mo, mm = m * m;
+    const long long n2 = (KG ? 4LL : 1LL) * pl.nmax * pl.nmax;
+    if (j < nat) {
+        sh.q[j] += f2d_steer(moved[j]);
+        sh.dq[j] = sh.q[j] - sh.zv[j];
+    }
+    __syncthreads();
+    if (a.n_disp > 0) return;   // a finite-difference copy needs only its charges
+    for (int kp = rank; kp < (KG ? pl.nk : 1); kp += blocks) {
+        const PState32 f = p_state32<KG>(wk, kp, n2, mm);
+        double *C = Cb + (KG ? (long long)kp * mm : 0);
+        fprod<5, 5, false, true>(sh, m, mo, mv, [&](int i, int k) { return f.C[(mo + k) * m + i]; },
+                                 [&](int k, int c) { return f.x[c * mv + k]; },
+                                 [&](int i, int c, float v) { C[(long long)c * m + i] += f2d_steer(v); });
+    }
+    if (!KG) {
+        const PState32 f = p_state32<KG>(wk, 0, n2, mm);
+        float *eo = (float *)sh.invd, *ea = (float *)sh.qst, *dA = (float *)wk.Mv;
+        if (j < nat) {
+            float s = 0.0f;
+            for (int k = 0; k < nat; ++k) s = fmaf(wk.g32[k * nat + j], moved[k], s);
+            ea[j] = 0.5f * s;
+        }
+        __syncthreads();
+        for (int i = j; i < m; i += PT) eo[i] = ea[sh.orb_atom[i]];
+        __syncthreads();
+        fprod<5, 5, true, true>(sh, mo, mo, m, [&](int i, int k) { return f.C[i * m + k]; },
+                                [&](int k, int c) { return eo[k] * f.SC[c * m + k]; },
+                                [&](int i, int c, float v) { dA[c * mo + i] = v; });
+    }
+    p_shifts(sh, pl, wk, nat);
+}
+
 // Warm-started cell: the method of k_water_warm and g_warm (dftb_kernel.cu, dftb_generic.cu) for the
 // staged products of this kernel and for a set of k-points coupled by the charges.
 //
@@ -437,7 +496,8 @@ __device__ __noinline__ void p_shifts(SH &sh, const PbcDev &pl, const PbcMem &w,
 // rule. Nothing of the FP32 part but the starting basis and the approximate Hessian enters the result.
 // The stored bases Cs are only read; the path works in Cb (wk.Cd). Returns false (in every block of the cell)
 // when the cell leaves the path's range, so that the general path starts from Cs. On success: Cb occupied
-// columns first (each block its own k-points), sh.q, sh.dq and sh.shift, and for the Gamma point Y = H C_o.
+// columns first (each block its own k-points), sh.q, sh.dq and sh.shift (not for a finite-difference copy), and
+// for the Gamma point Y = H C_o before the last change of the charges and in Mv (FP32) half of that change of A_oo.
 // Measured (GB300, one step): 304 cells of 33 waters 263 -> 76 ms (with the image lists and the Ewald split),
 // 24 cells of 8 waters on 3 x 3 x 3 232 -> 18.8 ms (with clusters of blocks); evaluations 11.8 -> 2.0. Bound: FP64
 // products (7.5 n^3 multiply-adds a cell) and pair sums, the pipe about 65 % busy.
@@ -456,17 +516,17 @@ __device__ __noinline__ bool p_warm(const DftbArgs &a, const PbcDev &pl, SH &sh,
     float *C32, *SC, *A32, *x, *r, *p, *hp;
     float wkp = 1.0f;
     auto set_k = [&](int kp) {
-        float *base = KG ? wk.kf + 4LL * kp * n2 : (float *)wk.P;
         if (KG) {
             H0 = wk.H0 + 2LL * kp * n2;
             S = H0 + n2;
             C = Cb + (long long)kp * mm;
             wkp = (float)pl.kpt[4 * kp + 3];
         }
-        C32 = base;
-        SC = base + mm;
-        A32 = KG ? base + 2 * mm : (float *)wk.Xg;
-        x = A32 + mm;   // K, residual, search direction and its image: n_virt n_occ <= m^2 / 4 each
+        const PState32 f = p_state32<KG>(wk, kp, n2, mm);
+        C32 = f.C;
+        SC = f.SC;
+        A32 = f.A;
+        x = f.x;   // K, residual, search direction and its image: n_virt n_occ <= m^2 / 4 each
         r = x + mvo;
         p = r + mvo;
         hp = p + mvo;
@@ -577,9 +637,11 @@ __device__ __noinline__ bool p_warm(const DftbArgs &a, const PbcDev &pl, SH &sh,
     auto diag_of = [&](int e) -> float { return A32[(mo + e % mv) * (m + 1)] - A32[(e / mv) * (m + 1)]; };
     // Hessian K = r (K in x, r destroyed) to a relative residual rel; false when it is not positive
     int steps = 0;   // conjugate-gradient steps of the last solve
+    float *moved = (float *)sh.hq[0];   // the change of the atoms' charges under K
     auto newton = [&](float rel) -> bool {
         float rz = 0.0f;
         steps = 0;
+        if (j < nat) moved[j] = 0.0f;
         for (int kp = rank; kp < NKP; kp += blocks) {
             set_k(kp);
             for (int e = j; e < mvo; e += PT) {
@@ -622,6 +684,7 @@ __device__ __noinline__ bool p_warm(const DftbArgs &a, const PbcDev &pl, SH &sh,
             ph = total(ph);
             if (!(ph > 0.0f)) return false;
             const float al = rz / ph;
+            if (j < nat) moved[j] = fmaf(al, dqf[j], moved[j]);
             float rn = 0.0f;
             for (int kp = rank; kp < NKP; kp += blocks) {
                 set_k(kp);
@@ -914,8 +977,9 @@ __device__ __noinline__ bool p_warm(const DftbArgs &a, const PbcDev &pl, SH &sh,
             build_a();
         }
         if (!all(finite)) return false;
+        bool conv = false;
+        float hi = -1e30f, lo = 1e30f;
         if (all(small)) {   // q_out - q to first order: K0 = r / (A_vv - A_oo)
-            float hi = -1e30f, lo = 1e30f;
             for (int kp = rank; kp < NKP; kp += blocks) {
                 set_k(kp);
                 for (int e = j; e < mvo; e += PT) x[e] = r[e] / diag_of(e);
@@ -924,69 +988,72 @@ __device__ __noinline__ bool p_warm(const DftbArgs &a, const PbcDev &pl, SH &sh,
             }
             __syncthreads();
             charges(0);
-            bool conv = true;
-            if (j < nat) conv = fabsf(dqf[j]) < (float)a.scc_tol;
-            if (all(conv)) {
-                // aufbau and gap over all k-points: tau - A_oo and A_vv - tau - PW_GAP positive definite for a tau
-                // between the highest occupied and the lowest empty diagonal (pivots of L D L^T)
-                if (blocks > 1) {
-                    double *mine = wk.xch + ((long long)parity * blocks + rank) * (pl.amax + 8);
-                    if (j == 0) {
-                        mine[0] = hi;
-                        mine[1] = lo;
-                    }
-                    cluster_barrier(blocks);
-                    for (int b = 0; b < blocks; ++b) {
-                        hi = fmaxf(hi, (float)__ldcg(wk.xch + ((long long)parity * blocks + b) * (pl.amax + 8)));
-                        lo = fminf(lo, (float)__ldcg(wk.xch + ((long long)parity * blocks + b) * (pl.amax + 8) + 1));
-                    }
-                    parity ^= 1;
+            conv = blk_all(j >= nat || fabsf(dqf[j]) < (float)a.scc_tol);   // the same charges in every block
+        }
+        if (conv) {
+            // aufbau and gap over all k-points: tau - A_oo and A_vv - tau - PW_GAP positive definite for a tau
+            // between the highest occupied and the lowest empty diagonal (pivots of L D L^T)
+            if (blocks > 1) {
+                double *mine = wk.xch + ((long long)parity * blocks + rank) * (pl.amax + 8);
+                if (j == 0) {
+                    mine[0] = hi;
+                    mine[1] = lo;
                 }
-                // the diagonals bound tau (mixing inside the blocks moves the levels beyond them): bisection
-                for (int t = 0;; ++t) {
-                    const float tau = 0.5f * (hi + lo);
-                    bool occ = true, emp = true;
-                    for (int kp = rank; kp < NKP; kp += blocks) {
-                        set_k(kp);
-                        // a row bound first: diagonally dominant rows are enough
-                        bool dom = true;
-                        for (int i = j; i < m; i += PT) {
-                            float off = 0.0f;
-                            const int b0 = i < mo ? 0 : mo, b1 = i < mo ? mo : m;
-                            for (int c = b0; c < b1; ++c)
-                                if (c != i) off += fabsf(A32[c * m + i]);
-                            const float d = i < mo ? tau - A32[i * (m + 1)] : A32[i * (m + 1)] - tau - PW_GAP;
-                            dom = dom && d > off;
-                        }
-                        if (blk_all(dom)) continue;
-                        for (int e = j; e < mm; e += PT) {
-                            const int c = e / m, i = e - c * m;
-                            T0[e] = (i < mo && c < mo) ? (i == c ? tau : 0.0f) - A32[e] : A32[e] - (i == c ? tau + PW_GAP : 0.0f);
+                cluster_barrier(blocks);
+                for (int b = 0; b < blocks; ++b) {
+                    hi = fmaxf(hi, (float)__ldcg(wk.xch + ((long long)parity * blocks + b) * (pl.amax + 8)));
+                    lo = fminf(lo, (float)__ldcg(wk.xch + ((long long)parity * blocks + b) * (pl.amax + 8) + 1));
+                }
+                parity ^= 1;
+            }
+            // the diagonals bound tau (mixing inside the blocks moves the levels beyond them): bisection
+            for (int t = 0;; ++t) {
+                const float tau = 0.5f * (hi + lo);
+                bool occ = true, emp = true;
+                for (int kp = rank; kp < NKP; kp += blocks) {
+                    set_k(kp);
+                    // a row bound first: diagonally dominant rows are enough
+                    bool dom = true;
+                    for (int i = j; i < m; i += PT) {
+                        float off = 0.0f;
+                        const int b0 = i < mo ? 0 : mo, b1 = i < mo ? mo : m;
+                        for (int c = b0; c < b1; ++c)
+                            if (c != i) off += fabsf(A32[c * m + i]);
+                        const float d = i < mo ? tau - A32[i * (m + 1)] : A32[i * (m + 1)] - tau - PW_GAP;
+                        dom = dom && d > off;
+                    }
+                    if (blk_all(dom)) continue;
+                    for (int e = j; e < mm; e += PT) {
+                        const int c = e / m, i = e - c * m;
+                        T0[e] = (i < mo && c < mo) ? (i == c ? tau : 0.0f) - A32[e] : A32[e] - (i == c ? tau + PW_GAP : 0.0f);
+                    }
+                    __syncthreads();
+                    for (int k = 0; k < m; ++k) {
+                        const float d = T0[k * (m + 1)];
+                        if (k < mo) occ = occ && d > 0.0f; else emp = emp && d > 0.0f;
+                        const int end = k < mo ? mo : m;
+                        const float id = 1.0f / d;
+                        for (int c = k + 1 + (j >> 5); c < end; c += PT / 32) {   // a warp per column of the trailing block
+                            const float f = T0[k * m + c] * id;
+                            for (int i = c + (j & 31); i < end; i += 32) T0[c * m + i] = fmaf(-f, T0[k * m + i], T0[c * m + i]);
                         }
                         __syncthreads();
-                        for (int k = 0; k < m; ++k) {
-                            const float d = T0[k * (m + 1)];
-                            if (k < mo) occ = occ && d > 0.0f; else emp = emp && d > 0.0f;
-                            const int end = k < mo ? mo : m;
-                            const float id = 1.0f / d;
-                            for (int c = k + 1 + (j >> 5); c < end; c += PT / 32) {   // a warp per column of the trailing block
-                                const float f = T0[k * m + c] * id;
-                                for (int i = c + (j & 31); i < end; i += 32) T0[c * m + i] = fmaf(-f, T0[k * m + i], T0[c * m + i]);
-                            }
-                            __syncthreads();
-                        }
                     }
-                    occ = all(occ);
-                    emp = all(emp);
-                    if (occ && emp) break;
-                    if (t == PW_BISECT || occ == emp) return false;
-                    if (occ) lo = tau; else hi = tau;
                 }
-                evals = it;
-                return true;
+                occ = all(occ);
+                emp = all(emp);
+                if (occ && emp) break;
+                if (t == PW_BISECT || occ == emp) return false;
+                if (occ) lo = tau; else hi = tau;
             }
         }
-        if (it == most || !newton(1e-7f)) return false;   // (1e-6 left one cell in ten above scc_tol)
+        // (a relative residual of 1e-6 left one cell in ten above scc_tol)
+        if ((it == most && !conv) || !newton(conv ? PW_LAST_TOL : 1e-7f)) return false;
+        if (conv) {
+            p_settle<KG>(a, pl, sh, wk, Cb, moved, n, nocc, nat, rank, blocks);
+            evals = it;
+            return true;
+        }
         float kmax = 0.0f;
         for (int kp = rank; kp < NKP; kp += blocks) {
             set_k(kp);
@@ -2107,7 +2174,10 @@ __device__ void p_cell(const DevSK &sk, const DftbArgs &a, const PbcDev &pl, SH 
         }
         pprod<true, true, true>(sh, nocc, nocc, n, [&](int o1, int k) { return C[sh.occ_list[o1] * n + k]; },
                                 [&](int k, int o2) { return Y[o2 * n + k]; },
-                                [&](int i, int c, double v) { Mo[c * nocc + i] = v; });
+                                [&](int i, int c, double v) {
+                                    const float *dA = (const float *)Mv;
+                                    Mo[c * nocc + i] = warm ? v + f2d_steer(dA[c * nocc + i] + dA[i * nocc + c]) : v;
+                                });
         pprod<false, false, false>(sh, nocc, n, nocc,
                                    [&](int o, int o2) { return Mo[min(o, o2) * nocc + max(o, o2)]; },
                                    [&](int o2, int c) { return C[sh.occ_list[o2] * n + c]; },

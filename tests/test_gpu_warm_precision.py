@@ -9,6 +9,7 @@ import pytest
 
 import cavmd_synth as cs
 from oracle import dftb as OD
+from oracle import periodic as PR
 
 pytestmark = pytest.mark.gpu
 
@@ -47,3 +48,19 @@ def test_clusters(P):
         s = slice(sy.cell_offset[c], sy.cell_offset[c + 1])
         ref = OD.dftb(pa, sy.species[s], st["r"][None, s], tol=2e-14, forces=False)
         assert np.abs(ev["q_pop"][s] - ref["q"][0]).max() < TOL
+
+
+def test_periodic_cells(P):
+    rng = np.random.default_rng(17)
+    cent = np.zeros((4, 3))
+    cent[:, 0] = 200.0 * np.arange(1, 5)
+    sy, lat = cs.periodic_water_cells(rng, cent, n_waters=33, side=10.0 * cs.ANGSTROM)
+    sy.p = cs.mb_momenta(rng, sy)
+    pa = cs.load_water_params()
+    ctx = P.Context(sy, pa, cs.line_modes(8, 1000.0, 0.001, k_max=0.01), lattice=lat)
+    ctx.cavmd_step(3)
+    ev, st = ctx.cavmd_get_eval(), ctx.cavmd_get_state()
+    for c in range(sy.n_cells):
+        s = slice(sy.cell_offset[c], sy.cell_offset[c + 1])
+        ref = PR.dftb_periodic(pa, sy.species[s], st["r"][s], lat, tol=2e-14, forces=False)
+        assert np.abs(ev["q_pop"][s] - ref["q"]).max() < TOL
