@@ -160,6 +160,13 @@ cudaError_t launch_tc_back(const TcPlan &p, const float *Wt2, const float *Wt1, 
 cudaError_t launch_tc_panels_com(const TcPlan &p, const double *r, const double *mass, const int *cell_offset,
                                  cudaStream_t st);
 
+// The larger operand, or NaN when either is one (fmaxf drops a NaN, and a bound tested on it would pass).
+__device__ __forceinline__ float max_nan(float a, float b) {
+    float r;
+    asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+    return r;
+}
+
 // Conversions between FP64 and FP32 on the integer pipe, for quantities that only steer an
 // iteration (generator entries, rotation angles, mixing coefficients): on GB300 the hardware
 // conversions issue to the FP64 pipe, the bottleneck of the SCC kernels. d2f_steer truncates the

@@ -37,7 +37,9 @@ constexpr int GW_FP32_ITERS = 5;       // warm path: bound on the FP32 Newton st
 constexpr float GW_FP32_KTOL = 3e-5f;  // the rotation below which the next step would be FP32 rounding
 constexpr float GW_ROT_MAX = 0.3f;     // the largest rotation taken (beyond: the general path)
 constexpr int GW_EVALS = 8;            // and bound on the FP64 evaluations
-constexpr float GW_ORTH_MAX = 1e-4f;   // overlap defect that the second-order correction takes
+constexpr float GW_ORTH_MAX = 5e-4f;   // norm of the overlap defect that the FP64 correction takes,
+constexpr float GW_ORTH_CUBE = 2e-5f;  // and above which its cubic term counts
+constexpr float GW_ROT64_MAX = 3e-4f;  // norm of a rotation between FP64 evaluations (C stays orthonormal to K^4 / 4)
 constexpr float GW_GAP = 2e-3f;        // HOMO-LUMO gap (Hartree) the warm path needs, above G_MIN_GAP
 constexpr int GW_CG_SLOW = 6;          // conjugate-gradient steps of the first Newton step that ask for a block sweep
 constexpr int GW_BISECT = 6;           // tries for a level between the occupied and the empty ones
@@ -263,7 +265,7 @@ struct GWarm {
 // (64 times the FP64 rate), each step solved by conjugate gradients on the orbital Hessian
 //   K -> A_vv K - K A_oo + C_v^T dH(K) C_o,  dH = S o (e_A + e_B) / 2, e = gamma dq(K),
 // preconditioned by the diagonal differences (3 to 7 iterations). Two steps reach FP32 rounding. Then
-// in FP64: the orthonormal correction C (1 - E/2 + 3/8 E^2); evaluations of q(C), H(q), H C_o and the
+// in FP64: the orthonormal correction C (1 - E/2 + 3/8 E^2 - 5/16 E^3); evaluations of q(C), H(q), H C_o and the
 // residual A_vo, each followed by the rotation C (1 + K + K^2/2) with K from the FP32 Hessian of this
 // basis. Converged when every |A_vo| < G_EIG_TOL and the populations that A_vo implies to first
 // order, q_out - q, are below scc_tol: two or three evaluations, about 9 n^3 FP64 multiply-adds with
@@ -452,6 +454,7 @@ __device__ bool g_warm(const DftbArgs &a, const GWarm &v, double *&C, double *&Y
                 rn = fmaf(q, q / diag_of(e), rn);
             }
             rn = sum(rn);
+            if (!(rn < 1e30f) || !(rn >= 0.0f)) return false;
             const float be = rn / rz;
             rz = rn;
             for (int e = j; e < nvo; e += T) p[e] = fmaf(be, p[e], r[e] / diag_of(e));
@@ -482,11 +485,11 @@ __device__ bool g_warm(const DftbArgs &a, const GWarm &v, double *&C, double *&Y
         float big = 0.0f;
         ftile<T, 3, 3>(j, n, n, n, F0, 1, LF, F1, LF, 1, [&](int i, int c, float t) {
             const float e = t - (i == c ? 1.0f : 0.0f);
-            big = fmaxf(big, fabsf(e));
+            big = max_nan(big, fabsf(e));
             if (pass == 0) F3[i * LF + c] = e;
             else F4[i * LF + c] = fmaf(-0.5f, e, i == c ? 1.0f : 0.0f);
         });
-        if (!all(big < 0.2f)) return false;   // NaN included
+        if (!all(big < 0.2f)) return false;   // a NaN too
         if (pass == 0) {
             g.sync();
             ftile<T, 3, 3>(j, n, n, n, F3, 1, LF, F3, LF, 1, [&](int i, int c, float t) {
@@ -529,7 +532,7 @@ __device__ bool g_warm(const DftbArgs &a, const GWarm &v, double *&C, double *&Y
         if (!newton(it < 2 ? 3e-3f : 1e-2f)) return false;
         if (it == 0) first_steps = steps;
         float kmax = 0.0f;
-        for (int e = j; e < nvo; e += T) kmax = fmaxf(kmax, fabsf(x[e]));
+        for (int e = j; e < nvo; e += T) kmax = max_nan(kmax, fabsf(x[e]));
         if (!all(kmax < GW_ROT_MAX)) return false;
         done = all(kmax < GW_FP32_KTOL);
         second(F4, true);
@@ -606,7 +609,7 @@ __device__ bool g_warm(const DftbArgs &a, const GWarm &v, double *&C, double *&Y
     g.sync();
     {   // E = C^T S C - 1 into A, and in FP32 into XB
         float *E32 = (float *)XB;
-        float big = 0.0f;
+        float e2 = 0.0f;
         flat<T, 4>(j, n * (n + 1) / 2, n, 1, 1,
                    [&](int e) { return C + g_lower(e, n).x * LD; },
                    [&](int e) { return Y + g_lower(e, n).y * LD; }, [&](int e, double t) {
@@ -618,15 +621,24 @@ __device__ bool g_warm(const DftbArgs &a, const GWarm &v, double *&C, double *&Y
                        const float f = d2f_steer(t);
                        E32[c * LF + i] = f;
                        E32[i * LF + c] = f;
-                       big = fmaxf(big, fabsf(f));
+                       e2 = fmaf(i == c ? 1.0f : 2.0f, f * f, e2);
                    });
-        if (!all(big < GW_ORTH_MAX)) return false;
+        e2 = sum(e2);
+        if (!(e2 < GW_ORTH_MAX * GW_ORTH_MAX)) return false;
         g.sync();
-        // 1 - E/2 + 3/8 E^2: E^2 is below 1e-8, so FP32 carries it beyond FP64 rounding
+        // 1 - E/2 + 3/8 E^2 - 5/16 E^3. The norm of E is 2e-6 as a rule, more after a large rotation; at its bound FP32
+        // rounds the last two terms by 6e-15, and the quartic one is 2e-14.
+        float *Q32 = (float *)Y;
         ftile<T, 3, 3>(j, n, n, n, E32, 1, LF, E32, LF, 1, [&](int i, int c, float t) {
             A[c * LD + i] = fma(-0.5, A[c * LD + i], (i == c ? 1.0 : 0.0) + f2d_steer(0.375f * t));
+            Q32[c * LF + i] = t;
         });
         g.sync();
+        if (e2 > GW_ORTH_CUBE * GW_ORTH_CUBE) {
+            ftile<T, 3, 3>(j, n, n, n, E32, 1, LF, Q32, 1, LF,
+                           [&](int i, int c, float t) { A[c * LD + i] -= f2d_steer(0.3125f * t); });
+            g.sync();
+        }
         flat<T, 4>(j, nn, n, LD, 1, [&](int e) { return C + (e % n); }, [&](int e) { return A + (e / n) * LD; },
                    [&](int e, double t) { Y[(e / n) * LD + e % n] = t; });
         g.sync();
@@ -746,9 +758,9 @@ __device__ bool g_warm(const DftbArgs &a, const GWarm &v, double *&C, double *&Y
             evals = it;
             return true;
         }
-        float kmax = 0.0f;
-        for (int e = j; e < nvo; e += T) kmax = fmaxf(kmax, fabsf(x[e]));
-        if (!all(kmax < 1e-2f)) return false;
+        float k2 = 0.0f;
+        for (int e = j; e < nvo; e += T) k2 = fmaf(x[e], x[e], k2);
+        if (!(sum(k2) < GW_ROT64_MAX * GW_ROT64_MAX)) return false;
         // C (1 + K + K^2/2), as C_o + (C_v - (C_o K^T)/2) K and C_v - (C_o + (C_v K)/2) K^T
         second(F1, false);
         double Kd[4];   // this thread's entries of K: n_virt n_occ <= n^2 / 4, 1024 on 256 threads at n = 64, 256 on 128 at n = 32

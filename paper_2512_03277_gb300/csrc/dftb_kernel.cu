@@ -32,7 +32,9 @@ constexpr int W_FP32_ITERS = 6;         // warm waters: bound on the FP32 Newton
 constexpr float W_FP32_KTOL = 1e-6f;    // the rotation at which they stop (FP32 rounding moves C by as much),
 constexpr float W_ROT_MAX = 0.3f;       // the largest rotation taken (beyond: the general solve)
 constexpr int W_EVALS = 8;              // and bound on the FP64 evaluations
-constexpr float W_ORTH_MAX = 1e-4f;     // overlap defect that the second-order correction takes
+constexpr float W_ORTH_MAX = 5e-4f;     // norm of the overlap defect that the FP64 correction takes,
+constexpr float W_ORTH_CUBE = 2e-5f;    // and above which its cubic term counts
+constexpr float W_ROT64_MAX = 3e-4f;    // norm of a rotation between FP64 evaluations
 constexpr float W_GAP = 2e-3f;          // HOMO-LUMO gap (Hartree) the warm path needs, above MIN_GAP
 
 // Scratch of one water in the warm path (k_water_warm). Matrices are row-major: the lane of orbital
@@ -995,7 +997,7 @@ __device__ __noinline__ void scc_general_water(const DftbArgs &a, MolShared<3, 6
 // runs in FP32: the previous basis is made S-orthonormal, then Newton steps on the orbital rotation
 // (the 8 occupied-virtual angles, with the charges' response, so that each step squares the error)
 // until the rotation reaches FP32 rounding. The FP64 part starts from that basis:
-//   C <- C (1 - E/2 + 3/8 E^2), E = C^T S C - 1 (about 1e-6 here, so orthonormal to 1e-18);
+//   C <- C (1 - E/2 + 3/8 E^2 - 5/16 E^3), E = C^T S C - 1 (about 1e-6 here);
 //   evaluations of the populations q(C), H(q) and the residual A_vo = C_v^T H C_o, all in FP64, each
 //   followed by the second-order rotation C (1 + K + K^2/2) with the Newton K of the last FP32
 //   Hessian (relative error about 1e-6, so the error falls by that factor).
@@ -1201,7 +1203,7 @@ __device__ __forceinline__ void water_warm(const DevSK &sk, const DftbArgs &a, c
 #pragma unroll
             for (int k = 0; k < 6; ++k) {
                 M[i][k] -= (i == k) ? 1.0f : 0.0f;
-                big = fmaxf(big, fabsf(M[i][k]));
+                big = max_nan(big, fabsf(M[i][k]));
             }
         ok = big < 0.2f;   // false for NaN
         // C (1 - E/2 + 3/8 E^2 - 5/16 E^3): E is a few 1e-2 after one step
@@ -1301,7 +1303,7 @@ __device__ __forceinline__ void water_warm(const DevSK &sk, const DftbArgs &a, c
         }
         float kmax = 0.0f;
 #pragma unroll
-        for (int i = 0; i < 8; ++i) kmax = fmaxf(kmax, fabsf(K[i]));
+        for (int i = 0; i < 8; ++i) kmax = max_nan(kmax, fabsf(K[i]));
         ok = ok && kmax < W_ROT_MAX;
         if (!done && ok) {   // a water that is done keeps its basis and Hessian whatever its warp does
             if (j == 0) {
@@ -1392,7 +1394,7 @@ __device__ __forceinline__ void water_warm(const DevSK &sk, const DftbArgs &a, c
         __syncwarp();
         double n[6];
         float ef[21], x1[6], x2[6];
-        float big = 0.0f;
+        float e2 = 0.0f;   // sum of (E/2)^2
 #pragma unroll
         for (int k = 0; k < 6; ++k) n[k] = c[k];
 #pragma unroll
@@ -1401,12 +1403,13 @@ __device__ __forceinline__ void water_warm(const DevSK &sk, const DftbArgs &a, c
             for (int q = 0; q <= p; ++q) {
                 const double e = w.E[p * (p + 1) / 2 + q];
                 ef[p * (p + 1) / 2 + q] = d2f_steer(e);
-                big = fmaxf(big, fabsf(ef[p * (p + 1) / 2 + q]));
+                e2 = fmaf(p == q ? 1.0f : 2.0f, ef[p * (p + 1) / 2 + q] * ef[p * (p + 1) / 2 + q], e2);
                 n[q] = fma(c[p], e, n[q]);
                 if (p != q) n[p] = fma(c[q], e, n[p]);
             }
-        ok = ok && big < W_ORTH_MAX;
-        // 3/8 E^2 = 3/2 (E/2)^2: below 1e-8, so FP32 carries it beyond FP64 rounding of C
+        ok = ok && 4.0f * e2 < W_ORTH_MAX * W_ORTH_MAX;
+        // 3/8 E^2 - 5/16 E^3, with H = -E/2: 3/2 H^2 + 5/2 H^3. The norm of E is 6e-7 as a rule and 1e-4 after a large
+        // rotation; at its bound FP32 rounds these terms by 6e-15, and the quartic one is 2e-14.
         auto efe = [&](const float *x, float *y) {
 #pragma unroll
             for (int q = 0; q < 6; ++q) {
@@ -1418,7 +1421,15 @@ __device__ __forceinline__ void water_warm(const DevSK &sk, const DftbArgs &a, c
         efe(cf, x1);
         efe(x1, x2);
 #pragma unroll
-        for (int k = 0; k < 6; ++k) c[k] = n[k] + f2d_steer(1.5f * x2[k]);
+        for (int k = 0; k < 6; ++k) x1[k] = 1.5f * x2[k];
+        if (__any_sync(CAVMD_FULL_MASK, 4.0f * e2 > W_ORTH_CUBE * W_ORTH_CUBE)) {
+            float x3[6];
+            efe(x2, x3);
+#pragma unroll
+            for (int k = 0; k < 6; ++k) x1[k] = fmaf(2.5f, x3[k], x1[k]);
+        }
+#pragma unroll
+        for (int k = 0; k < 6; ++k) c[k] = n[k] + f2d_steer(x1[k]);
     }
     put_C();
 
@@ -1493,7 +1504,7 @@ __device__ __forceinline__ void water_warm(const DevSK &sk, const DftbArgs &a, c
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
             rhs[i] = w.av[i];
-            amax = fmaxf(amax, fabsf(rhs[i]));
+            amax = max_nan(amax, fabsf(rhs[i]));
         }
         w_solve(L, rhs, K);
 #pragma unroll
@@ -1505,10 +1516,14 @@ __device__ __forceinline__ void water_warm(const DevSK &sk, const DftbArgs &a, c
         if (!conv && ok) {
             used = it;
             conv = amax < (float)EIG_TOL && move < tol;
-            ok = amax < 1.0f;   // false for NaN
+            float k2 = 0.0f;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) k2 = fmaf(K[i], K[i], k2);
+            ok = amax < 1.0f && k2 < W_ROT64_MAX * W_ROT64_MAX;   // false for NaN
         }
         if (__all_sync(CAVMD_FULL_MASK, conv || !ok || !act)) break;
-        if (!conv && ok && it < evals) {   // the rotation; its second-order part is below FP32 rounding of the first
+        if (!conv && ok && it < evals) {   // the rotation; its second-order part in FP32: of a norm below 5e-8,
+                                              // so rounded below 3e-15; and C stays orthonormal to K^4 / 4 < 3e-15
             float sv[2], ro[4], c32[6];
 #pragma unroll
             for (int k = 0; k < 6; ++k) c32[k] = d2f_steer(c[k]);

@@ -56,7 +56,9 @@ constexpr int PW_FP32_ITERS = 5;        // warm path (p_warm): bound on the FP32
 constexpr float PW_FP32_KTOL = 3e-5f;   // the rotation below which the next step would be FP32 rounding
 constexpr float PW_ROT_MAX = 0.3f;      // the largest rotation taken (beyond: the general path)
 constexpr int PW_EVALS = 8;             // and bound on the FP64 evaluations
-constexpr float PW_ORTH_MAX = 1e-4f;    // overlap defect that the second-order correction takes
+constexpr float PW_ORTH_MAX = 5e-4f;    // norm (over all k-points) of the overlap defect that the FP64 correction takes,
+constexpr float PW_ORTH_CUBE = 2e-5f;   // the norm (of one k-point) above which its cubic term counts,
+constexpr float PW_ROT64_MAX = 3e-4f;   // and norm of a rotation between FP64 evaluations (C stays orthonormal to K^4 / 4)
 constexpr float PW_GAP = 2e-3f;         // HOMO-LUMO gap (Hartree) the warm path needs, above P_MIN_GAP
 constexpr int PW_CG_SLOW = 6;           // conjugate-gradient steps of the first Newton step that ask for a block sweep
 constexpr int PW_BISECT = 6;            // tries for a level between the occupied and the empty ones
@@ -490,7 +492,7 @@ __device__ __noinline__ void p_settle(const DftbArgs &a, const PbcDev &pl, SH &s
 // orthonormal and moved by Newton steps of the orbital rotation in FP32, 64 times the FP64 rate; each
 // step is solved by conjugate gradients over all k-points (inner product weighted like the energy) on
 //   K_k -> A_vv K_k - K_k A_oo + C_v^T dH_k C_o,  dH = S o (e_A + e_B) / 2, e = gamma sum_k w_k dq(K_k).
-// Then in FP64: C (1 - E/2 + 3/8 E^2), evaluations of q(C), H, H C_o and the residual A_vo, each followed
+// Then in FP64: C (1 - E/2 + 3/8 E^2 - 5/16 E^3), evaluations of q(C), H, H C_o and the residual A_vo, each followed
 // by C (1 + K + K^2/2) with K from the FP32 Hessian of this basis; converged when every |A_vo| < P_EIG_TOL
 // and the populations that A_vo implies to first order, q_out - q, are below scc_tol: two evaluations as a
 // rule. Nothing of the FP32 part but the starting basis and the approximate Hessian enters the result.
@@ -696,6 +698,7 @@ __device__ __noinline__ bool p_warm(const DftbArgs &a, const PbcDev &pl, SH &sh,
                 }
             }
             rn = total(rn);
+            if (!(rn < 1e30f) || !(rn >= 0.0f)) return false;
             const float be = rn / rz;
             rz = rn;
             for (int kp = rank; kp < NKP; kp += blocks) {
@@ -749,8 +752,7 @@ __device__ __noinline__ bool p_warm(const DftbArgs &a, const PbcDev &pl, SH &sh,
             fprod<7, 7, true, true>(sh, m, m, m, [&](int i, int k) { return C32[i * m + k]; },
                                     [&](int k, int c) { return SC[c * m + k]; }, [&](int i, int c, float v) {
                                         const float e = v - (i == c ? 1.0f : 0.0f);
-                                        big = fmaxf(big, fabsf(e));
-                                        if (!(big < 1e30f)) big = 1e30f;
+                                        big = max_nan(big, fabsf(e));
                                         if (pass == 0) T0[c * m + i] = e;
                                         else T1[c * m + i] = fmaf(-0.5f, e, i == c ? 1.0f : 0.0f);
                                     });
@@ -801,7 +803,7 @@ __device__ __noinline__ bool p_warm(const DftbArgs &a, const PbcDev &pl, SH &sh,
         float kmax = 0.0f;
         for (int kp = rank; kp < NKP; kp += blocks) {
             set_k(kp);
-            for (int e = j; e < mvo; e += PT) kmax = fmaxf(kmax, fabsf(x[e]));
+            for (int e = j; e < mvo; e += PT) kmax = max_nan(kmax, fabsf(x[e]));
             second(true);
             fprod<5, 5, false, true>(sh, m, mo, mv, [&](int i, int k) { return T1[(mo + k) * m + i]; },
                                      [&](int k, int c) { return x[c * mv + k]; },
@@ -875,9 +877,10 @@ __device__ __noinline__ bool p_warm(const DftbArgs &a, const PbcDev &pl, SH &sh,
     }
 
     // ---------------------------------------------------------------- FP64: orthonormal bases
-    big = 0.0f;
+    float e2 = 0.0f;
     for (int kp = rank; kp < NKP; kp += blocks) {
         set_k(kp);
+        float ek = 0.0f;   // this thread's share of the k-point's sum
         for (int e = j; e < mm; e += PT) C[e] = f2d_steer(C32[e]);
         __syncthreads();
         auto Cat = [&](int i, int c) -> double { return C[(long long)c * m + i]; };
@@ -891,21 +894,28 @@ __device__ __noinline__ bool p_warm(const DftbArgs &a, const PbcDev &pl, SH &sh,
                                     const float f = d2f_steer(v);
                                     T0[c * m + i] = f;
                                     T0[i * m + c] = f;
-                                    big = fmaxf(big, fabsf(f));
+                                    ek = fmaf(i == c ? 1.0f : 2.0f, f * f, ek);
                                 });
-        // 1 - E/2 + 3/8 E^2: E^2 is below 1e-8, so FP32 carries it beyond FP64 rounding
+        // 1 - E/2 + 3/8 E^2 - 5/16 E^3. The norm of E is 2e-6 (36 waters: 7e-6, 14 k-points: 2e-5) as a rule, more after a
+        // large rotation; at its bound FP32 rounds the last two terms by 6e-15, and the quartic one is 2e-14.
         fprod<7, 7, false, true>(sh, m, m, m, [&](int i, int k) { return T0[k * m + i]; },
                                  [&](int k, int c) { return T0[c * m + k]; }, [&](int i, int c, float v) {
                                      double &h = H[(long long)c * m + i];
                                      h = fma(-0.5, h, (i == c ? 1.0 : 0.0) + f2d_steer(0.375f * v));
+                                     T1[c * m + i] = v;
                                  });
+        e2 += ek;
+        if (!blk_all(ek * PT < PW_ORTH_CUBE * PW_ORTH_CUBE))   // then the sum is below it too
+            fprod<7, 7, false, true>(sh, m, m, m, [&](int i, int k) { return T0[k * m + i]; },
+                                     [&](int k, int c) { return T1[c * m + k]; },
+                                     [&](int i, int c, float v) { H[(long long)c * m + i] -= f2d_steer(0.3125f * v); });
         pprod<false, false, true>(sh, m, m, m, [&](int i, int k) { return C[(long long)k * m + i]; },
                                   [&](int k, int c) { return H[(long long)c * m + k]; },
                                   [&](int i, int c, double v) { Y[(long long)c * m + i] = v; });
         for (int e = j; e < mm; e += PT) C[e] = Y[e];
         __syncthreads();
     }
-    if (!all(big < PW_ORTH_MAX)) return false;
+    if (!(total(e2) < PW_ORTH_MAX * PW_ORTH_MAX)) return false;
 
     // ---------------------------------------------------------------- FP64 evaluations
     const int most = min(a.max_iter, PW_EVALS);
@@ -1054,12 +1064,12 @@ __device__ __noinline__ bool p_warm(const DftbArgs &a, const PbcDev &pl, SH &sh,
             evals = it;
             return true;
         }
-        float kmax = 0.0f;
+        float k2 = 0.0f;
         for (int kp = rank; kp < NKP; kp += blocks) {
             set_k(kp);
-            for (int e = j; e < mvo; e += PT) kmax = fmaxf(kmax, fabsf(x[e]));
+            for (int e = j; e < mvo; e += PT) k2 = fmaf(x[e], x[e], k2);
         }
-        if (!all(kmax < 1e-2f)) return false;
+        if (!(total(k2) < PW_ROT64_MAX * PW_ROT64_MAX)) return false;
         for (int kp = rank; kp < NKP; kp += blocks) {
             set_k(kp);
             // C (1 + K + K^2/2), as C_o + (C_v - (C_o K^T)/2) K and C_v - (C_o + (C_v K)/2) K^T; the half terms in FP32

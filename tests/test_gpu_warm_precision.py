@@ -64,3 +64,21 @@ def test_periodic_cells(P):
         s = slice(sy.cell_offset[c], sy.cell_offset[c + 1])
         ref = PR.dftb_periodic(pa, sy.species[s], st["r"][s], lat, tol=2e-14, forces=False)
         assert np.abs(ev["q_pop"][s] - ref["q"]).max() < TOL
+
+
+def test_fast_waters_keep_their_electrons(P):
+    """Momenta 2.5 times and a time step twice as large: rotations at the edge of the warm path leave the
+    largest overlap defects E that it takes. The populations of a water sum to 2 tr(C_o^T S C_o) = 8.
+
+    Tolerance: with the norm of E below 5e-4, what the correction leaves out (35/128 E^4) is below 1.7e-14
+    and FP32 rounds its last terms by 6e-15: 2 sqrt(4) 2.3e-14 on the trace, and 1e-14 for the sums."""
+    w = cs.make_workload("c2", n_cells=4000, n_modes=16)
+    w["system"].p *= 2.5
+    o = P.default_options()
+    o.dt *= 2.0
+    ctx = P.Context(w["system"], w["params"], w["modes"], o)
+    ctx.cavmd_step(1)
+    ev = ctx.cavmd_get_eval()
+    warm = ev["scc_iters"] <= 4
+    assert warm.sum() > 100
+    assert np.abs(ev["q_pop"].reshape(-1, 3).sum(1) - 8.0)[warm].max() < 1.02e-13
