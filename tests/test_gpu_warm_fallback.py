@@ -1,9 +1,11 @@
-"""Cells that leave the warm-started path, beside others that stay on it, against the oracles at the context's own positions. Tolerances: those of the parity tests
+"""Cells that leave the warm-started path, beside others that stay on it, and the widest k-point
+problems, against the oracles at the context's own positions. Tolerances: those of the parity tests
 (forces 1e-9 of the largest, populations and cell energies 1e-10)."""
 import numpy as np
 import pytest
 
 import cavmd_synth as cs
+from oracle import dftb as OD
 from oracle import periodic as PR
 
 pytestmark = pytest.mark.gpu
@@ -66,3 +68,36 @@ def test_periodic_cells_that_leave_the_warm_path(P, grid):
         it = _check(ctx, sy, _solver(pa, lat, grid))
         if step == 0:
             assert it.max() > 4 > it.min()   # both ways were taken
+
+
+def test_clusters_that_leave_the_warm_path(P):
+    rng = np.random.default_rng(7)
+    sizes = [6, 1, 8, 2, 3, 10, 4]
+    sy = cs.cluster_batch(rng, sizes, np.zeros((len(sizes), 3)))
+    sy.p = cs.mb_momenta(rng, sy)
+    sy.p *= np.repeat(np.where(np.arange(len(sizes)) % 2 == 0, 3.0, 1.0), np.diff(sy.cell_offset))[:, None]
+    o = P.default_options()
+    o.dt *= 2.0
+    pa = cs.load_water_params()
+    ctx = P.Context(sy, pa, cs.line_modes(8, 1000.0, 0.001, k_max=0.01), o)
+
+    def solve(sp, r):
+        ref = OD.dftb(pa, sp, r[None])
+        return {k: ref[k][0] for k in ("F", "q", "E")}
+
+    for step in range(2):
+        ctx.cavmd_step(1)
+        it = _check(ctx, sy, solve)
+        if step == 0:
+            assert it.max() > 4 > it.min()
+
+
+def test_warm_steps_of_wide_k_points(P):
+    """Twenty-two waters, 132 orbitals: real forms of 264 rows, beyond the 256 of the smaller kernel."""
+    sy, lat = _periodic(22, 2)
+    o = P.default_options()
+    o.kgrid[:] = (2, 1, 1)
+    pa = cs.load_water_params()
+    ctx = P.Context(sy, pa, cs.line_modes(8, 1000.0, 0.001, k_max=0.01), o, lattice=lat)
+    ctx.cavmd_step(2)
+    assert _check(ctx, sy, _solver(pa, lat, (2, 1, 1))).max() <= 4
