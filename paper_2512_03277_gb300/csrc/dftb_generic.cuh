@@ -37,9 +37,11 @@ constexpr int GW_FP32_ITERS = 5;       // warm path: bound on the FP32 Newton st
 constexpr float GW_FP32_KTOL = 3e-5f;  // the rotation below which the next step would be FP32 rounding
 constexpr float GW_ROT_MAX = 0.3f;     // the largest rotation taken (beyond: the general path)
 constexpr int GW_EVALS = 8;            // and bound on the FP64 evaluations
-constexpr float GW_ORTH_MAX = 5e-4f;   // norm of the overlap defect that the FP64 correction takes,
+constexpr float GW_ORTH_MAX = 3e-2f;   // norm of the overlap defect that the FP64 correction takes,
+constexpr float GW_ORTH_ONCE = 5e-4f;  // above which it is repeated
 constexpr float GW_ORTH_CUBE = 2e-5f;  // and above which its cubic term counts
-constexpr float GW_ROT64_MAX = 3e-4f;  // norm of a rotation between FP64 evaluations (C stays orthonormal to K^4 / 4)
+constexpr float GW_ROT64_MAX = 1e-2f;  // norm of a rotation between FP64 evaluations,
+constexpr float GW_ROT64_ONCE = 3e-4f; // and above which the correction follows it (below, C stays orthonormal to 3e-15)
 constexpr float GW_GAP = 2e-3f;        // HOMO-LUMO gap (Hartree) the warm path needs, above G_MIN_GAP
 constexpr int GW_CG_SLOW = 6;          // conjugate-gradient steps of the first Newton step that ask for a block sweep
 constexpr int GW_BISECT = 6;           // tries for a level between the occupied and the empty ones
@@ -597,61 +599,64 @@ __device__ bool g_warm(const DftbArgs &a, const GWarm &v, double *&C, double *&Y
         }
     }
 
-    // ---------------------------------------------------------------- FP64: orthonormal basis
+    // ---------------------------------------------------------------- FP64 evaluations
     for (int e = j; e < nn; e += T) {
         const int c = e / n, i = e - c * n;
         C[c * LD + i] = f2d_steer(F0[i * LF + c]);
-        A[c * LD + i] = s_at(i, c);
     }
-    g.sync();
-    flat<T, 4>(j, nn, n, LD, 1, [&](int e) { return A + (e % n); }, [&](int e) { return C + (e / n) * LD; },
-               [&](int e, double t) { Y[(e / n) * LD + e % n] = t; });
-    g.sync();
-    {   // E = C^T S C - 1 into A, and in FP32 into XB
-        float *E32 = (float *)XB;
-        float e2 = 0.0f;
-        flat<T, 4>(j, n * (n + 1) / 2, n, 1, 1,
-                   [&](int e) { return C + g_lower(e, n).x * LD; },
-                   [&](int e) { return Y + g_lower(e, n).y * LD; }, [&](int e, double t) {
-                       const int2 ic = g_lower(e, n);
-                       const int i = ic.x, c = ic.y;
-                       if (i == c) t -= 1.0;
-                       A[c * LD + i] = t;
-                       A[i * LD + c] = t;
-                       const float f = d2f_steer(t);
-                       E32[c * LF + i] = f;
-                       E32[i * LF + c] = f;
-                       e2 = fmaf(i == c ? 1.0f : 2.0f, f * f, e2);
-                   });
-        e2 = sum(e2);
-        if (!(e2 < GW_ORTH_MAX * GW_ORTH_MAX)) return false;
-        g.sync();
-        // 1 - E/2 + 3/8 E^2 - 5/16 E^3. The norm of E is 2e-6 as a rule, more after a large rotation; at its bound FP32
-        // rounds the last two terms by 6e-15, and the quartic one is 2e-14.
-        float *Q32 = (float *)Y;
-        ftile<T, 3, 3>(j, n, n, n, E32, 1, LF, E32, LF, 1, [&](int i, int c, float t) {
-            A[c * LD + i] = fma(-0.5, A[c * LD + i], (i == c ? 1.0 : 0.0) + f2d_steer(0.375f * t));
-            Q32[c * LF + i] = t;
-        });
-        g.sync();
-        if (e2 > GW_ORTH_CUBE * GW_ORTH_CUBE) {
-            ftile<T, 3, 3>(j, n, n, n, E32, 1, LF, Q32, 1, LF,
-                           [&](int i, int c, float t) { A[c * LD + i] -= f2d_steer(0.3125f * t); });
-            g.sync();
-        }
-        flat<T, 4>(j, nn, n, LD, 1, [&](int e) { return C + (e % n); }, [&](int e) { return A + (e / n) * LD; },
-                   [&](int e, double t) { Y[(e / n) * LD + e % n] = t; });
-        g.sync();
-        double *t = C;
-        C = Y;
-        Y = t;
-        F0 = (float *)Y;
-        F1 = F0 + n * LF;
-    }
-
-    // ---------------------------------------------------------------- FP64 evaluations
+    bool rough = true;   // the basis is orthonormal to FP32 only (or after a large rotation)
     const int most = min(a.max_iter, GW_EVALS);
     for (int it = 1; it <= most; ++it) {
+        for (int pass = 0; rough; ++pass) {
+            for (int e = j; e < nn; e += T) {
+                const int c = e / n, i = e - c * n;
+                A[c * LD + i] = s_at(i, c);
+            }
+            g.sync();
+            flat<T, 4>(j, nn, n, LD, 1, [&](int e) { return A + (e % n); }, [&](int e) { return C + (e / n) * LD; },
+                       [&](int e, double t) { Y[(e / n) * LD + e % n] = t; });
+            g.sync();
+            // E = C^T S C - 1 into A, and in FP32 into XB
+            float *E32 = (float *)XB, *Q32 = (float *)Y;
+            float e2 = 0.0f;
+            flat<T, 4>(j, n * (n + 1) / 2, n, 1, 1,
+                       [&](int e) { return C + g_lower(e, n).x * LD; },
+                       [&](int e) { return Y + g_lower(e, n).y * LD; }, [&](int e, double t) {
+                           const int2 ic = g_lower(e, n);
+                           const int i = ic.x, c = ic.y;
+                           if (i == c) t -= 1.0;
+                           A[c * LD + i] = t;
+                           A[i * LD + c] = t;
+                           const float f = d2f_steer(t);
+                           E32[c * LF + i] = f;
+                           E32[i * LF + c] = f;
+                           e2 = fmaf(i == c ? 1.0f : 2.0f, f * f, e2);
+                       });
+            e2 = sum(e2);
+            if (!(e2 < GW_ORTH_MAX * GW_ORTH_MAX) || pass == 3) return false;
+            rough = e2 > GW_ORTH_ONCE * GW_ORTH_ONCE;
+            g.sync();
+            // 1 - E/2 + 3/8 E^2 - 5/16 E^3. The norm of E is 2e-6 as a rule, more after a large rotation; up to
+            // GW_ORTH_ONCE FP32 rounds the last two terms by 6e-15, and the quartic one is 2e-14.
+            ftile<T, 3, 3>(j, n, n, n, E32, 1, LF, E32, LF, 1, [&](int i, int c, float t) {
+                A[c * LD + i] = fma(-0.5, A[c * LD + i], (i == c ? 1.0 : 0.0) + f2d_steer(0.375f * t));
+                Q32[c * LF + i] = t;
+            });
+            g.sync();
+            if (e2 > GW_ORTH_CUBE * GW_ORTH_CUBE) {
+                ftile<T, 3, 3>(j, n, n, n, E32, 1, LF, Q32, 1, LF,
+                               [&](int i, int c, float t) { A[c * LD + i] -= f2d_steer(0.3125f * t); });
+                g.sync();
+            }
+            flat<T, 4>(j, nn, n, LD, 1, [&](int e) { return C + (e % n); }, [&](int e) { return A + (e / n) * LD; },
+                       [&](int e, double t) { Y[(e / n) * LD + e % n] = t; });
+            g.sync();
+            double *t = C;
+            C = Y;
+            Y = t;
+        }
+        F0 = (float *)Y;
+        F1 = F0 + n * LF;
         for (int e = j; e < nn; e += T) {
             const int c = e / n, i = e - c * n;
             A[c * LD + i] = s_at(i, c);
@@ -760,7 +765,9 @@ __device__ bool g_warm(const DftbArgs &a, const GWarm &v, double *&C, double *&Y
         }
         float k2 = 0.0f;
         for (int e = j; e < nvo; e += T) k2 = fmaf(x[e], x[e], k2);
-        if (!(sum(k2) < GW_ROT64_MAX * GW_ROT64_MAX)) return false;
+        k2 = sum(k2);
+        if (!(k2 < GW_ROT64_MAX * GW_ROT64_MAX)) return false;
+        rough = k2 > GW_ROT64_ONCE * GW_ROT64_ONCE;
         // C (1 + K + K^2/2), as C_o + (C_v - (C_o K^T)/2) K and C_v - (C_o + (C_v K)/2) K^T
         second(F1, false);
         double Kd[4];   // this thread's entries of K: n_virt n_occ <= n^2 / 4, 1024 on 256 threads at n = 64, 256 on 128 at n = 32

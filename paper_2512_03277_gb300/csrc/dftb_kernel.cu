@@ -32,9 +32,11 @@ constexpr int W_FP32_ITERS = 6;         // warm waters: bound on the FP32 Newton
 constexpr float W_FP32_KTOL = 1e-6f;    // the rotation at which they stop (FP32 rounding moves C by as much),
 constexpr float W_ROT_MAX = 0.3f;       // the largest rotation taken (beyond: the general solve)
 constexpr int W_EVALS = 8;              // and bound on the FP64 evaluations
-constexpr float W_ORTH_MAX = 5e-4f;     // norm of the overlap defect that the FP64 correction takes,
+constexpr float W_ORTH_MAX = 3e-2f;     // norm of the overlap defect that the FP64 correction takes,
+constexpr float W_ORTH_ONCE = 5e-4f;    // above which it is repeated
 constexpr float W_ORTH_CUBE = 2e-5f;    // and above which its cubic term counts
-constexpr float W_ROT64_MAX = 3e-4f;    // norm of a rotation between FP64 evaluations
+constexpr float W_ROT64_MAX = 1e-2f;    // norm of a rotation between FP64 evaluations,
+constexpr float W_ROT64_ONCE = 3e-4f;   // and above which the correction follows it
 constexpr float W_GAP = 2e-3f;          // HOMO-LUMO gap (Hartree) the warm path needs, above MIN_GAP
 
 // Scratch of one water in the warm path (k_water_warm). Matrices are row-major: the lane of orbital
@@ -1360,78 +1362,6 @@ __device__ __forceinline__ void water_warm(const DevSK &sk, const DftbArgs &a, c
         for (int i = 0; i < 8; ++i) w.B[(j - 4) * 8 + i] = bh[i];
     }
     put_C();
-    {
-        double x[6];
-#pragma unroll
-        for (int k = 0; k < 6; ++k) x[k] = 0.0;
-#pragma unroll
-        for (int i = 0; i < 6; ++i) {
-            const double2 *row = reinterpret_cast<const double2 *>(w.C + 6 * i);
-#pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                const double2 v = row[k];
-                x[2 * k] = fma(sr[i], v.x, x[2 * k]);
-                x[2 * k + 1] = fma(sr[i], v.y, x[2 * k + 1]);
-            }
-        }
-        if (act) {
-            double2 *row = reinterpret_cast<double2 *>(w.X + 6 * j);
-            row[0] = make_double2(x[0], x[1]);
-            row[1] = make_double2(x[2], x[3]);
-            row[2] = make_double2(x[4], x[5]);
-        }
-        __syncwarp();
-        if (act) {   // -E/2, entry (p, q), p >= q, at p (p + 1) / 2 + q: 21 entries over 6 lanes
-            for (int e = j; e < 21; e += 6) {
-                int p = (e >= 15) ? 5 : (e >= 10) ? 4 : (e >= 6) ? 3 : (e >= 3) ? 2 : (e >= 1) ? 1 : 0;
-                const int q = e - p * (p + 1) / 2;
-                double s = p == q ? -1.0 : 0.0;
-#pragma unroll
-                for (int i = 0; i < 6; ++i) s = fma(w.C[6 * i + p], w.X[6 * i + q], s);
-                w.E[e] = -0.5 * s;
-            }
-        }
-        __syncwarp();
-        double n[6];
-        float ef[21], x1[6], x2[6];
-        float e2 = 0.0f;   // sum of (E/2)^2
-#pragma unroll
-        for (int k = 0; k < 6; ++k) n[k] = c[k];
-#pragma unroll
-        for (int p = 0; p < 6; ++p)
-#pragma unroll
-            for (int q = 0; q <= p; ++q) {
-                const double e = w.E[p * (p + 1) / 2 + q];
-                ef[p * (p + 1) / 2 + q] = d2f_steer(e);
-                e2 = fmaf(p == q ? 1.0f : 2.0f, ef[p * (p + 1) / 2 + q] * ef[p * (p + 1) / 2 + q], e2);
-                n[q] = fma(c[p], e, n[q]);
-                if (p != q) n[p] = fma(c[q], e, n[p]);
-            }
-        ok = ok && 4.0f * e2 < W_ORTH_MAX * W_ORTH_MAX;
-        // 3/8 E^2 - 5/16 E^3, with H = -E/2: 3/2 H^2 + 5/2 H^3. The norm of E is 6e-7 as a rule and 1e-4 after a large
-        // rotation; at its bound FP32 rounds these terms by 6e-15, and the quartic one is 2e-14.
-        auto efe = [&](const float *x, float *y) {
-#pragma unroll
-            for (int q = 0; q < 6; ++q) {
-                y[q] = 0.0f;
-#pragma unroll
-                for (int p = 0; p < 6; ++p) y[q] = fmaf(x[p], p >= q ? ef[p * (p + 1) / 2 + q] : ef[q * (q + 1) / 2 + p], y[q]);
-            }
-        };
-        efe(cf, x1);
-        efe(x1, x2);
-#pragma unroll
-        for (int k = 0; k < 6; ++k) x1[k] = 1.5f * x2[k];
-        if (__any_sync(CAVMD_FULL_MASK, 4.0f * e2 > W_ORTH_CUBE * W_ORTH_CUBE)) {
-            float x3[6];
-            efe(x2, x3);
-#pragma unroll
-            for (int k = 0; k < 6; ++k) x1[k] = fmaf(2.5f, x3[k], x1[k]);
-        }
-#pragma unroll
-        for (int k = 0; k < 6; ++k) c[k] = n[k] + f2d_steer(x1[k]);
-    }
-    put_C();
 
     // ---------------------------------------------------------------- FP64 evaluations
     double q0 = 0.0, q1 = 0.0, q2 = 0.0, s0 = 0.0, s1 = 0.0, s2 = 0.0;   // populations of one spin, half shifts
@@ -1484,7 +1414,87 @@ __device__ __forceinline__ void water_warm(const DevSK &sk, const DftbArgs &a, c
     bool conv = false;
     int used = 0;
     float K[8], move1 = 0.0f, move2 = 0.0f;   // the rotation that the last residual asks for, the charges' change under it
+    bool rough = act && ok;   // the basis is orthonormal to FP32 only (or after a large rotation)
     for (int it = 1; it <= evals; ++it) {
+        for (int pass = 0; pass < 3 && __any_sync(CAVMD_FULL_MASK, rough); ++pass) {
+            double x[6];
+#pragma unroll
+            for (int k = 0; k < 6; ++k) x[k] = 0.0;
+#pragma unroll
+            for (int i = 0; i < 6; ++i) {
+                const double2 *row = reinterpret_cast<const double2 *>(w.C + 6 * i);
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    const double2 v = row[k];
+                    x[2 * k] = fma(sr[i], v.x, x[2 * k]);
+                    x[2 * k + 1] = fma(sr[i], v.y, x[2 * k + 1]);
+                }
+            }
+            if (act) {
+                double2 *row = reinterpret_cast<double2 *>(w.X + 6 * j);
+                row[0] = make_double2(x[0], x[1]);
+                row[1] = make_double2(x[2], x[3]);
+                row[2] = make_double2(x[4], x[5]);
+            }
+            __syncwarp();
+            if (act) {   // -E/2, entry (p, q), p >= q, at p (p + 1) / 2 + q: 21 entries over 6 lanes
+                for (int e = j; e < 21; e += 6) {
+                    int p = (e >= 15) ? 5 : (e >= 10) ? 4 : (e >= 6) ? 3 : (e >= 3) ? 2 : (e >= 1) ? 1 : 0;
+                    const int q = e - p * (p + 1) / 2;
+                    double s = p == q ? -1.0 : 0.0;
+#pragma unroll
+                    for (int i = 0; i < 6; ++i) s = fma(w.C[6 * i + p], w.X[6 * i + q], s);
+                    w.E[e] = -0.5 * s;
+                }
+            }
+            __syncwarp();
+            double n[6];
+            float ef[21], x0[6], x1[6], x2[6];
+            float e2 = 0.0f;   // sum of (E/2)^2
+#pragma unroll
+            for (int k = 0; k < 6; ++k) n[k] = c[k];
+#pragma unroll
+            for (int p = 0; p < 6; ++p)
+#pragma unroll
+                for (int q = 0; q <= p; ++q) {
+                    const double e = w.E[p * (p + 1) / 2 + q];
+                    ef[p * (p + 1) / 2 + q] = d2f_steer(e);
+                    e2 = fmaf(p == q ? 1.0f : 2.0f, ef[p * (p + 1) / 2 + q] * ef[p * (p + 1) / 2 + q], e2);
+                    n[q] = fma(c[p], e, n[q]);
+                    if (p != q) n[p] = fma(c[q], e, n[p]);
+                }
+            // 3/8 E^2 - 5/16 E^3, with H = -E/2: 3/2 H^2 + 5/2 H^3. The norm of E is 6e-7 as a rule, more after a large
+            // rotation; up to W_ORTH_ONCE FP32 rounds these terms by 6e-15, and the quartic one is 2e-14.
+            auto efe = [&](const float *x, float *y) {
+#pragma unroll
+                for (int q = 0; q < 6; ++q) {
+                    y[q] = 0.0f;
+#pragma unroll
+                    for (int p = 0; p < 6; ++p) y[q] = fmaf(x[p], p >= q ? ef[p * (p + 1) / 2 + q] : ef[q * (q + 1) / 2 + p], y[q]);
+                }
+            };
+#pragma unroll
+            for (int k = 0; k < 6; ++k) x0[k] = d2f_steer(c[k]);
+            efe(x0, x1);
+            efe(x1, x2);
+#pragma unroll
+            for (int k = 0; k < 6; ++k) x1[k] = 1.5f * x2[k];
+            if (4.0f * e2 > W_ORTH_CUBE * W_ORTH_CUBE) {
+                float x3[6];
+                efe(x2, x3);
+#pragma unroll
+                for (int k = 0; k < 6; ++k) x1[k] = fmaf(2.5f, x3[k], x1[k]);
+            }
+            if (rough) {   // the others of the warp keep their basis to the bit
+#pragma unroll
+                for (int k = 0; k < 6; ++k) c[k] = n[k] + f2d_steer(x1[k]);
+                ok = ok && 4.0f * e2 < W_ORTH_MAX * W_ORTH_MAX;   // false for NaN
+                rough = ok && 4.0f * e2 > W_ORTH_ONCE * W_ORTH_ONCE;
+            }
+            put_C();
+        }
+        ok = ok && !rough;
+        rough = false;
         evaluate();
         if (act) {
             for (int e = j; e < 8; e += 6) {
@@ -1520,10 +1530,11 @@ __device__ __forceinline__ void water_warm(const DevSK &sk, const DftbArgs &a, c
 #pragma unroll
             for (int i = 0; i < 8; ++i) k2 = fmaf(K[i], K[i], k2);
             ok = amax < 1.0f && k2 < W_ROT64_MAX * W_ROT64_MAX;   // false for NaN
+            rough = ok && !conv && k2 > W_ROT64_ONCE * W_ROT64_ONCE;
         }
         if (__all_sync(CAVMD_FULL_MASK, conv || !ok || !act)) break;
-        if (!conv && ok && it < evals) {   // the rotation; its second-order part in FP32: of a norm below 5e-8,
-                                              // so rounded below 3e-15; and C stays orthonormal to K^4 / 4 < 3e-15
+        if (!conv && ok && it < evals) {   // the rotation; its second-order part in FP32: up to W_ROT64_ONCE of a
+                                              // norm below 5e-8, rounded below 3e-15, and C stays orthonormal to K^4 / 4 < 3e-15
             float sv[2], ro[4], c32[6];
 #pragma unroll
             for (int k = 0; k < 6; ++k) c32[k] = d2f_steer(c[k]);

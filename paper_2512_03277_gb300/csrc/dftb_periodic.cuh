@@ -56,9 +56,11 @@ constexpr int PW_FP32_ITERS = 5;        // warm path (p_warm): bound on the FP32
 constexpr float PW_FP32_KTOL = 3e-5f;   // the rotation below which the next step would be FP32 rounding
 constexpr float PW_ROT_MAX = 0.3f;      // the largest rotation taken (beyond: the general path)
 constexpr int PW_EVALS = 8;             // and bound on the FP64 evaluations
-constexpr float PW_ORTH_MAX = 5e-4f;    // norm (over all k-points) of the overlap defect that the FP64 correction takes,
-constexpr float PW_ORTH_CUBE = 2e-5f;   // the norm (of one k-point) above which its cubic term counts,
-constexpr float PW_ROT64_MAX = 3e-4f;   // and norm of a rotation between FP64 evaluations (C stays orthonormal to K^4 / 4)
+constexpr float PW_ORTH_MAX = 5e-4f;    // norm (over all k-points) of the overlap defect that the last FP64 correction takes,
+constexpr float PW_ORTH_ONCE = 5e-4f;   // norm (of one k-point) above which another one follows
+constexpr float PW_ORTH_CUBE = 2e-5f;   // and above which its cubic term counts
+constexpr float PW_ROT64_MAX = 1e-2f;   // norm of a rotation between FP64 evaluations,
+constexpr float PW_ROT64_ONCE = 3e-4f;  // and above which the correction follows it (below, C stays orthonormal to 3e-15)
 constexpr float PW_GAP = 2e-3f;         // HOMO-LUMO gap (Hartree) the warm path needs, above P_MIN_GAP
 constexpr int PW_CG_SLOW = 6;           // conjugate-gradient steps of the first Newton step that ask for a block sweep
 constexpr int PW_BISECT = 6;            // tries for a level between the occupied and the empty ones
@@ -876,50 +878,61 @@ __device__ __noinline__ bool p_warm(const DftbArgs &a, const PbcDev &pl, SH &sh,
         }
     }
 
-    // ---------------------------------------------------------------- FP64: orthonormal bases
-    float e2 = 0.0f;
+    // ---------------------------------------------------------------- FP64 evaluations
     for (int kp = rank; kp < NKP; kp += blocks) {
         set_k(kp);
-        float ek = 0.0f;   // this thread's share of the k-point's sum
         for (int e = j; e < mm; e += PT) C[e] = f2d_steer(C32[e]);
-        __syncthreads();
-        auto Cat = [&](int i, int c) -> double { return C[(long long)c * m + i]; };
-        pprod<false, false, true>(sh, m, m, m, [&](int i, int k) { return S[(long long)k * m + i]; }, Cat,
-                                  [&](int i, int c, double v) { Y[(long long)c * m + i] = v; });
-        pprod<true, true, true>(sh, m, m, m, [&](int i, int k) { return C[(long long)i * m + k]; },
-                                [&](int k, int c) { return Y[(long long)c * m + k]; }, [&](int i, int c, double v) {
-                                    if (i == c) v -= 1.0;
-                                    H[(long long)c * m + i] = v;
-                                    H[(long long)i * m + c] = v;
-                                    const float f = d2f_steer(v);
-                                    T0[c * m + i] = f;
-                                    T0[i * m + c] = f;
-                                    ek = fmaf(i == c ? 1.0f : 2.0f, f * f, ek);
-                                });
-        // 1 - E/2 + 3/8 E^2 - 5/16 E^3. The norm of E is 2e-6 (36 waters: 7e-6, 14 k-points: 2e-5) as a rule, more after a
-        // large rotation; at its bound FP32 rounds the last two terms by 6e-15, and the quartic one is 2e-14.
-        fprod<7, 7, false, true>(sh, m, m, m, [&](int i, int k) { return T0[k * m + i]; },
-                                 [&](int k, int c) { return T0[c * m + k]; }, [&](int i, int c, float v) {
-                                     double &h = H[(long long)c * m + i];
-                                     h = fma(-0.5, h, (i == c ? 1.0 : 0.0) + f2d_steer(0.375f * v));
-                                     T1[c * m + i] = v;
-                                 });
-        e2 += ek;
-        if (!blk_all(ek * PT < PW_ORTH_CUBE * PW_ORTH_CUBE))   // then the sum is below it too
-            fprod<7, 7, false, true>(sh, m, m, m, [&](int i, int k) { return T0[k * m + i]; },
-                                     [&](int k, int c) { return T1[c * m + k]; },
-                                     [&](int i, int c, float v) { H[(long long)c * m + i] -= f2d_steer(0.3125f * v); });
-        pprod<false, false, true>(sh, m, m, m, [&](int i, int k) { return C[(long long)k * m + i]; },
-                                  [&](int k, int c) { return H[(long long)c * m + k]; },
-                                  [&](int i, int c, double v) { Y[(long long)c * m + i] = v; });
-        for (int e = j; e < mm; e += PT) C[e] = Y[e];
-        __syncthreads();
     }
-    if (!(total(e2) < PW_ORTH_MAX * PW_ORTH_MAX)) return false;
-
-    // ---------------------------------------------------------------- FP64 evaluations
+    __syncthreads();
+    bool rough = true;   // the bases are orthonormal to FP32 only (or after a large rotation)
     const int most = min(a.max_iter, PW_EVALS);
     for (int it = 1; it <= most; ++it) {
+        if (rough) {
+            float e2 = 0.0f;
+            for (int kp = rank; kp < NKP; kp += blocks) {
+                set_k(kp);
+                bool again = true;
+                for (int pass = 0; again; ++pass) {
+                    float ek = 0.0f;   // this thread's share of the k-point's sum
+                    pprod<false, false, true>(sh, m, m, m, [&](int i, int k) { return S[(long long)k * m + i]; },
+                                              [&](int i, int c) { return C[(long long)c * m + i]; },
+                                              [&](int i, int c, double v) { Y[(long long)c * m + i] = v; });
+                    pprod<true, true, true>(sh, m, m, m, [&](int i, int k) { return C[(long long)i * m + k]; },
+                                            [&](int k, int c) { return Y[(long long)c * m + k]; },
+                                            [&](int i, int c, double v) {
+                                                if (i == c) v -= 1.0;
+                                                H[(long long)c * m + i] = v;
+                                                H[(long long)i * m + c] = v;
+                                                const float f = d2f_steer(v);
+                                                T0[c * m + i] = f;
+                                                T0[i * m + c] = f;
+                                                ek = fmaf(i == c ? 1.0f : 2.0f, f * f, ek);
+                                            });
+                    // (a bound on every share bounds the sum)
+                    again = pass < 2 && !blk_all(ek * PT < PW_ORTH_ONCE * PW_ORTH_ONCE);
+                    if (!again) e2 += ek;
+                    // 1 - E/2 + 3/8 E^2 - 5/16 E^3. The norm of E is 2e-6 (36 waters: 7e-6, 14 k-points: 2e-5) as a
+                    // rule, more after a large rotation; up to PW_ORTH_ONCE FP32 rounds the last two terms by 6e-15,
+                    // and the quartic one is 2e-14.
+                    fprod<7, 7, false, true>(sh, m, m, m, [&](int i, int k) { return T0[k * m + i]; },
+                                             [&](int k, int c) { return T0[c * m + k]; }, [&](int i, int c, float v) {
+                                                 double &h = H[(long long)c * m + i];
+                                                 h = fma(-0.5, h, (i == c ? 1.0 : 0.0) + f2d_steer(0.375f * v));
+                                                 T1[c * m + i] = v;
+                                             });
+                    if (!blk_all(ek * PT < PW_ORTH_CUBE * PW_ORTH_CUBE))
+                        fprod<7, 7, false, true>(sh, m, m, m, [&](int i, int k) { return T0[k * m + i]; },
+                                                 [&](int k, int c) { return T1[c * m + k]; },
+                                                 [&](int i, int c, float v) { H[(long long)c * m + i] -= f2d_steer(0.3125f * v); });
+                    pprod<false, false, true>(sh, m, m, m, [&](int i, int k) { return C[(long long)k * m + i]; },
+                                              [&](int k, int c) { return H[(long long)c * m + k]; },
+                                              [&](int i, int c, double v) { Y[(long long)c * m + i] = v; });
+                    for (int e = j; e < mm; e += PT) C[e] = Y[e];
+                    __syncthreads();
+                }
+            }
+            if (!(total(e2) < PW_ORTH_MAX * PW_ORTH_MAX)) return false;
+        }
         // populations: 2 sum_o C(i, o) (S C)(i, o), weighted over the k-points
         for (int i = j; i < n; i += PT) sh.qk[i] = 0.0;
         __syncthreads();
@@ -1069,7 +1082,9 @@ __device__ __noinline__ bool p_warm(const DftbArgs &a, const PbcDev &pl, SH &sh,
             set_k(kp);
             for (int e = j; e < mvo; e += PT) k2 = fmaf(x[e], x[e], k2);
         }
-        if (!(total(k2) < PW_ROT64_MAX * PW_ROT64_MAX)) return false;
+        k2 = total(k2);
+        if (!(k2 < PW_ROT64_MAX * PW_ROT64_MAX)) return false;
+        rough = k2 > PW_ROT64_ONCE * PW_ROT64_ONCE;
         for (int kp = rank; kp < NKP; kp += blocks) {
             set_k(kp);
             // C (1 + K + K^2/2), as C_o + (C_v - (C_o K^T)/2) K and C_v - (C_o + (C_v K)/2) K^T; the half terms in FP32
