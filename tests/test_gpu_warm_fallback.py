@@ -101,30 +101,3 @@ def test_warm_steps_of_wide_k_points(P):
     ctx = P.Context(sy, pa, cs.line_modes(8, 1000.0, 0.001, k_max=0.01), o, lattice=lat)
     ctx.cavmd_step(2)
     assert _check(ctx, sy, _solver(pa, lat, (2, 1, 1))).max() <= 4
-
-
-def test_a_water_does_not_depend_on_its_warp(P):
-    """Waters of very different speeds share warps; without coupling each gives, to the bit, what it gives alone."""
-    n = 30
-    w = cs.make_workload("c2", n_cells=n, n_modes=8)
-    sy = w["system"]
-    sy.p *= np.repeat(np.tile([0.3, 1.0, 2.0, 2.5, 4.0], n // 5), 3)[:, None]
-    w["modes"].lam = 0.0 * w["modes"].lam
-    o = P.default_options()
-    o.dt *= 2.0
-
-    def run(s, r, p, R):
-        one = cs.System(species=sy.species[s], cell_offset=np.arange(0, len(r) + 1, 3, dtype=np.int32), r=r, p=p, R_ref=R)
-        ctx = P.Context(one, w["params"], w["modes"], o)
-        ctx.cavmd_step(1)
-        return ctx.cavmd_get_eval()
-
-    every = slice(0, 3 * n)
-    together = run(every, sy.r.copy(), sy.p.copy(), sy.R_ref)
-    assert together["scc_iters"].max() > 4 > together["scc_iters"].min()
-    for c in range(n):
-        s = slice(3 * c, 3 * c + 3)
-        alone = run(s, sy.r[s].copy(), sy.p[s].copy(), sy.R_ref[c:c + 1])
-        assert np.array_equal(alone["q_pop"], together["q_pop"][s])
-        assert np.array_equal(alone["F_dftb"].reshape(-1, 3), together["F_dftb"].reshape(-1, 3)[s])
-        assert alone["E_cell"][0] == together["E_cell"][c]
