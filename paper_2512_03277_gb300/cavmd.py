@@ -293,7 +293,10 @@ class Context:
             self.opt.stream = C.c_void_p(stream_handle)
 
             def _alloc(nbytes, user):
-                return torch.cuda.caching_allocator_alloc(int(nbytes), dev, self._torch_stream)
+                try:
+                    return torch.cuda.caching_allocator_alloc(int(nbytes), dev, self._torch_stream)
+                except torch.cuda.OutOfMemoryError:   # the library takes less where it can, else CAVMD_ERR_NOMEM
+                    return 0
 
             def _free(ptr, user):
                 torch.cuda.caching_allocator_delete(ptr)

@@ -998,8 +998,15 @@ int build_context(cavmd_ctx *c, const cavmd_system *sys, const cavmd_sk_tables *
         AL(pp.d_img, img.size());
         AL(pp.d_gw, gw.size());
         AL(pp.d_gi, gi.size());
-        AL(pp.work, pbc_workspace_doubles(pp.nmax, pp.amax, pp.n_g, pp.g_max, nk, pp.cluster) * (size_t)pp.blocks);
+        // where the allocator has not the memory for all the cells that could be in flight, fewer are
+        for (int rc; (rc = dalloc_n(c, &pp.work, pbc_workspace_doubles(pp))) != CAVMD_OK;) {
+            cudaGetLastError();
+            if (rc != CAVMD_ERR_NOMEM || !shrink_dftb_periodic(pp)) return rc;
+            c->err.clear();
+        }
         if (nk > 0) {
+            const size_t rows = c->n_disp > 0 ? (size_t)disp_per_atom * pp.amax : 1;
+            if (pp.cluster > 1) AL(pp.late, 1 + (size_t)N * rows);
             AL(pp.d_kpt, kpts.size());
             CK(cudaMemcpyAsync(pp.d_kpt, kpts.data(), sizeof(double) * kpts.size(), cudaMemcpyHostToDevice, st));
         }

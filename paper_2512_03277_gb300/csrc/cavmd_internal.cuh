@@ -271,12 +271,16 @@ struct PbcPlan {
                                           // r_cut); half-space reciprocal vectors
     int nmax, amax;                       // largest cell
     int blocks, cluster;                  // cells in flight; blocks that share a cell (k-grid; else 1)
+    int alone;                            // k-grid: cells in flight at one block each (cold starts, late cells)
+    int *late;                            // k-grid, clusters of blocks: device [1 + items], the count and the items
+                                          // (cells, finite-difference copies) that left the warm path
     double *d_img, *d_gw;                 // device: [n_img][3], [n_g][4] (G, 2 w_G)
-    double *work;                         // device: per-block workspaces
+    double *work;                         // device: the workspaces of the cells in flight
     int nk;                               // k-grid: irreducible k-points (0: Gamma point only)
     double *d_kpt;                        // device: [nk][4] fractional k and weight
 };
-size_t pbc_workspace_doubles(int nmax, int amax, int n_g, int g_max, int nk, int cluster);
+size_t pbc_workspace_doubles(const PbcPlan &p);   // of all cells in flight
+bool shrink_dftb_periodic(PbcPlan &p);            // halves the cells in flight; false when one is left
 const void *pbc_kg_small();   // the k-grid kernels (problems up to 256 and up to 512 wide)
 const void *pbc_kg_large();
 std::vector<double> pbc_kpoints(const int *kgrid);

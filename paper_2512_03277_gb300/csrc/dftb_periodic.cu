@@ -16,7 +16,7 @@ __global__ void __launch_bounds__(PT, 2) k_dftb_periodic(const DevSK *__restrict
     const int rows = pbc_rows(a, pl);
     for (long long it = blockIdx.x; it < (long long)rows * a.n_cells; it += gridDim.x) {
         int cell, row;
-        if (pbc_item(a, rows, it, cell, row)) p_cell<false>(*skp, a, pl, sh, wk, cell, row, 0, 1);
+        if (pbc_item(a, rows, it, cell, row)) p_cell<false>(*skp, a, pl, sh, wk, cell, row, 0, 1, 0);
     }
 }
 
@@ -25,10 +25,29 @@ __global__ void __launch_bounds__(PT, 2) k_dftb_periodic(const DevSK *__restrict
 // ---------------------------------------------------------------------------------------------
 // Host side
 
-size_t pbc_workspace_doubles(int nmax, int amax, int n_g, int g_max, int nk, int cluster) {
-    const size_t n2 = (nk > 0 ? 4 : 1) * (size_t)nmax * nmax, k = nk > 0 ? nk : 1, a2 = (size_t)amax * amax;
-    const size_t own = 6 * n2 + 2 * (size_t)n_g + 4 * a2 + (a2 + 1) / 2 + 6 * (size_t)amax * (g_max + 1) + 1;
-    return (nk > 0 ? 5 : 3) * k * n2 + a2 + 2 * (size_t)amax * n_g + 2 * (size_t)cluster * (amax + 8) + cluster * own + 32;
+namespace {
+
+// Doubles of one cell's workspace (pbc_mem) for `cluster` blocks; lean: without the warm path's FP32 state and
+// working bases.
+size_t pbc_cell_doubles(const PbcPlan &p, int cluster, bool lean) {
+    const size_t n2 = (p.nk > 0 ? 4 : 1) * (size_t)p.nmax * p.nmax, k = p.nk > 0 ? p.nk : 1, a2 = (size_t)p.amax * p.amax;
+    const size_t own = 6 * n2 + 2 * (size_t)p.n_g + 4 * a2 + (a2 + 1) / 2 + 6 * (size_t)p.amax * (p.g_max + 1) + 1;
+    return (lean ? 2 : p.nk > 0 ? 5 : 3) * k * n2 + a2 + 2 * (size_t)p.amax * p.n_g + 2 * (size_t)cluster * (p.amax + 8) +
+           cluster * own + 32;
+}
+
+}  // namespace
+
+size_t pbc_workspace_doubles(const PbcPlan &p) {
+    const size_t warm = pbc_cell_doubles(p, p.cluster, false) * p.blocks;
+    return p.nk > 0 ? std::max(warm, pbc_cell_doubles(p, 1, true) * p.alone) : warm;
+}
+
+bool shrink_dftb_periodic(PbcPlan &p) {
+    if (p.blocks == 1 && (p.nk <= 0 || p.alone == 1)) return false;
+    p.blocks = (p.blocks + 1) / 2;
+    p.alone = (p.alone + 1) / 2;
+    return true;
 }
 
 // The irreducible points of a Gamma-centred n1 x n2 x n3 grid: k and -k (modulo the reciprocal
@@ -183,8 +202,12 @@ cudaError_t kg_clusters(int nmax, int c, int *n) {
 // the chip idle a cluster of blocks shares each: the size that gives the fewest rounds of k-points,
 // ceil(nk / c) ceil(n_cells / resident clusters of c), the smaller one on a tie (24 cells on 3 x 3 x 3:
 // 14 points on 24 blocks before).
+// A cold start takes the general path, one block per cell and SM, and so do cells that leave the warm path of a
+// cluster: these are listed and evaluated by a launch of their own, so that no cluster's other blocks wait for them.
 cudaError_t plan_dftb_periodic_launch(PbcPlan &p, int n_cells, int n_sm) {
     p.cluster = 1;
+    p.alone = std::max(1, std::min(n_cells, n_sm));
+    p.late = nullptr;
     if (p.nk <= 0) {
         p.blocks = std::max(1, std::min(n_cells, 2 * n_sm));
         return cudaSuccess;
@@ -203,9 +226,11 @@ cudaError_t plan_dftb_periodic_launch(PbcPlan &p, int n_cells, int n_sm) {
         }
     }
     if (best < 0) return cudaErrorInvalidConfiguration;
-    // dense grids of large cells: at most 128 GiB of workspace, the blocks taking several cells in turn
-    const size_t each = 8 * pbc_workspace_doubles(p.nmax, p.amax, p.n_g, p.g_max, p.nk, p.cluster);
-    p.blocks = (int)std::max<size_t>(1, std::min<size_t>(p.blocks, ((size_t)128 << 30) / each));
+    // dense grids of large cells: at most 128 GiB of workspace, the blocks taking several cells in turn (and less
+    // when the allocator has less: shrink_dftb_periodic)
+    const size_t most = ((size_t)128 << 30) / 8;
+    p.blocks = (int)std::max<size_t>(1, std::min<size_t>(p.blocks, most / pbc_cell_doubles(p, p.cluster, false)));
+    p.alone = (int)std::max<size_t>(1, std::min<size_t>(p.alone, most / pbc_cell_doubles(p, 1, true)));
     return cudaSuccess;
 }
 
@@ -238,29 +263,45 @@ cudaError_t launch_dftb_periodic(const DevSK *sk_dev, const DftbArgs &a, const P
     d.img = p.d_img;
     d.gw = p.d_gw;
     d.work = p.work;
-    d.work_stride = (long long)pbc_workspace_doubles(p.nmax, p.amax, p.n_g, p.g_max, p.nk, p.cluster);
     d.nk = p.nk;
     d.cluster = p.cluster;
     d.kpt = p.d_kpt;
+    d.late = nullptr;
+    d.late_pass = d.lean = 0;
+    d.work_stride = (long long)pbc_cell_doubles(p, p.cluster, false);
     const long long items = a.n_disp > 0 ? (long long)a.n_cells * (a.fd_central ? 6 : 3) * p.amax : a.n_cells;
     const int groups = (int)std::min<long long>(items, p.blocks);
     if (p.nk > 0) {
-        // a cold start (the general path, one block per cell) takes the wider kernel's registers
-        const bool cold = !a.have_warm;
-        if (cold) d.cluster = 1;
-        cudaLaunchConfig_t cfg = {};
-        cudaLaunchAttribute at[1];
-        cfg.gridDim = dim3(groups * d.cluster);
-        cfg.blockDim = dim3(PT);
-        cfg.dynamicSmemBytes = kg_smem(cold ? PNMAX : p.nmax);
-        cfg.stream = st;
-        at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = d.cluster;
-        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-        cfg.attrs = at;
-        cfg.numAttrs = 1;
-        void *args[] = {(void *)&sk_dev, (void *)&a, (void *)&d};
-        return cudaLaunchKernelExC(&cfg, kg_kernel(cold ? PNMAX : p.nmax), args);
+        auto run = [&](int n, int nmax) {
+            cudaLaunchConfig_t cfg = {};
+            cudaLaunchAttribute at[1];
+            cfg.gridDim = dim3(n * d.cluster);
+            cfg.blockDim = dim3(PT);
+            cfg.dynamicSmemBytes = kg_smem(nmax);
+            cfg.stream = st;
+            at[0].id = cudaLaunchAttributeClusterDimension;
+            at[0].val.clusterDim.x = d.cluster;
+            at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+            cfg.attrs = at;
+            cfg.numAttrs = 1;
+            void *args[] = {(void *)&sk_dev, (void *)&a, (void *)&d};
+            return cudaLaunchKernelExC(&cfg, kg_kernel(nmax), args);
+        };
+        if (a.have_warm) {
+            if (p.cluster == 1) return run(groups, p.nmax);
+            d.late = p.late;
+            cudaError_t e = cudaMemsetAsync(p.late, 0, sizeof(int), st);
+            if (e == cudaSuccess) e = run(groups, p.nmax);
+            if (e != cudaSuccess) return e;
+            d.late_pass = 1;
+        }
+        // the general path, one block per cell with the wider kernel's registers: a cold start, or the late cells
+        // (a finite-difference copy needs the working bases)
+        d.cluster = 1;
+        d.lean = a.n_disp == 0;
+        d.work_stride = (long long)pbc_cell_doubles(p, 1, d.lean);
+        const long long room = (long long)pbc_workspace_doubles(p) / d.work_stride;
+        return run((int)std::min({items, room, (long long)p.alone}), PNMAX);
     }
     k_dftb_periodic<<<groups, PT, sizeof(PShared), st>>>(sk_dev, a, d);
     return cudaGetLastError();

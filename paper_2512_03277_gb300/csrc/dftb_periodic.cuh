@@ -290,6 +290,9 @@ struct PbcDev {
     long long work_stride;       // doubles per block
     int nk;                      // k-grid: irreducible k-points (0: Gamma-point kernel)
     int cluster;                 // k-grid: blocks that share a cell
+    int lean;                    // k-grid: workspaces without the warm path's part
+    int late_pass;               // k-grid: 1 evaluates the items of `late` by the general path
+    int *late;                   // k-grid, clusters: [1 + items] count and items that left the warm path
     const double *kpt;           // [nk][4] fractional k (units of the reciprocal rows) and weight
 };
 
@@ -1164,10 +1167,11 @@ __device__ __forceinline__ void pbc_pair(const SH &sh, int nat, int t, int &A, i
 // and the forces use the real-space densities rho(T) = sum_k w_k Re[P(k)_{nu mu} exp(i 2 pi f_k . n_T)]
 // (and the same for the energy-weighted density) image by image.
 // `blocks` blocks (a cluster; one outside the k-grid) share the cell: each takes the k-points rank,
-// rank + blocks, ... of the build, the warm path and the forces; the general path is rank 0's alone.
+// rank + blocks, ... A cluster only takes the warm path: a cell that leaves it puts its item on the list pl.late
+// and returns.
 template <bool KG, class SH>
 __device__ void p_cell(const DevSK &sk, const DftbArgs &a, const PbcDev &pl, SH &sh, const PbcMem &wk, int cell,
-                       int disp_k, int rank, int blocks) {
+                       int disp_k, int rank, int blocks, int item) {
     const int j = threadIdx.x;
     const int a0 = a.cell_offset[cell];
     const int nat = a.cell_offset[cell + 1] - a0;
@@ -1493,14 +1497,15 @@ __device__ void p_cell(const DevSK &sk, const DftbArgs &a, const PbcDev &pl, SH 
     // ---------------------------------------------------------------- warm path
     bool warm = false;
     int evals = 0;
-    if (a.have_warm && mo > 0 && m > mo) {
+    if (a.have_warm && mo > 0 && m > mo && !(KG && pl.late_pass)) {
         warm = p_warm<KG>(a, pl, sh, wk, C0, wk.Cd, n, nocc, nat, rank, blocks, evals);
         if (j < nat) sh.qst[j] = a.qpop[a0 + j];
         if (j == 0) sh.fl[2] = evals;
         __syncthreads();
     }
-    if (!warm && rank > 0) {   // the general path is rank 0's
-        cluster_barrier(blocks);
+    if (!warm && blocks > 1) {
+        if (rank == 0 && j == 0) pl.late[1 + atomicAdd(pl.late, 1)] = item;
+        cluster_barrier(blocks);   // the workspace is the next cell's from here on
         return;
     }
     if (warm) {
@@ -1937,7 +1942,6 @@ __device__ void p_cell(const DevSK &sk, const DftbArgs &a, const PbcDev &pl, SH 
     }
     __syncthreads();
     }   // general path
-    const int parts = warm ? blocks : 1;   // blocks that evaluate the forces (k-points rank, rank + parts, ...)
     if (disp) {   // a finite-difference copy: only its dipole
         if (j == 0 && rank == 0) {
             double mu[3] = {0.0, 0.0, 0.0};
@@ -1985,8 +1989,7 @@ __device__ void p_cell(const DevSK &sk, const DftbArgs &a, const PbcDev &pl, SH 
         }
         double eb_t = 0.0;   // this thread's part of the band energy sum_k w_k Re Tr P(k) H0(k)*
         const double rc2 = sk.r_cut * sk.r_cut;
-        const bool mine = rank < parts;
-        for (int kp = rank; kp < NKP && mine; kp += parts) {
+        for (int kp = rank; kp < NKP; kp += blocks) {
             set_k(kp);
             const bool first = kp == 0, fresh = kp == rank;
             const double wkp = pl.kpt[4 * kp + 3];
@@ -2170,16 +2173,16 @@ __device__ void p_cell(const DevSK &sk, const DftbArgs &a, const PbcDev &pl, SH 
             sh.red[0] = eb;
             if (rank > 0) sgf[0] = eb;   // (the structure factors are rank 0's to read from here on)
         }
-        if (parts > 1) {   // rank 0 adds the others' gradients and band energies, in rank order
+        if (blocks > 1) {   // rank 0 adds the others' gradients and band energies, in rank order
             cluster_barrier(blocks);
             if (rank == 0) {
                 const long long apart = wk.pbuf_stride;
                 for (int e = j; e < nat * nat; e += PT)
                     if (e / nat <= e % nat)
-                        for (int b = 1; b < min(parts, NKP); ++b)
+                        for (int b = 1; b < min(blocks, NKP); ++b)
                             for (int k = 0; k < 3; ++k) pbuf[4LL * e + k] += __ldcg(pbuf + b * apart + 4LL * e + k);
                 if (j == 0)
-                    for (int b = 1; b < parts; ++b) sh.red[0] += __ldcg(sgf + b * apart);
+                    for (int b = 1; b < blocks; ++b) sh.red[0] += __ldcg(sgf + b * apart);
             }
         }
         for (int r = j; r < n; r += PT)
@@ -2428,10 +2431,11 @@ __device__ __forceinline__ PbcMem pbc_mem(const PbcDev &pl, bool kg, long long g
     w.S = p + n2;
     p += 2 * nk * n2;
     w.kf = (float *)p;
-    if (kg) p += 2 * nk * n2;
+    if (kg && !pl.lean) p += 2 * nk * n2;
     w.gam = p; p += a2;
     w.csg = p; p += 2LL * pl.amax * pl.n_g;
-    w.Cd = p; p += nk * n2;
+    w.Cd = p;
+    if (!pl.lean) p += nk * n2;
     w.xch = p; p += 2LL * blocks * (pl.amax + 8);
     const long long own = 6 * n2 + 2LL * pl.n_g + 4 * a2 + (a2 + 1) / 2 + 6LL * pl.amax * (pl.g_max + 1) + 1;
     p += rank * own;
@@ -2454,9 +2458,11 @@ __global__ void __launch_bounds__(PT, MB) k_dftb_periodic_kg(const DevSK *__rest
     const int rank = pl.cluster > 1 ? (int)cluster_rank() : 0, group = blockIdx.x / pl.cluster;
     const PbcMem wk = pbc_mem(pl, true, group, rank, pl.cluster);
     const int rows = pbc_rows(a, pl);
-    for (long long it = group; it < (long long)rows * a.n_cells; it += gridDim.x / pl.cluster) {
+    const long long items = pl.late_pass ? pl.late[0] : (long long)rows * a.n_cells;
+    for (long long at = group; at < items; at += gridDim.x / pl.cluster) {
+        const long long it = pl.late_pass ? pl.late[1 + at] : at;
         int cell, row;
-        if (pbc_item(a, rows, it, cell, row)) p_cell<true>(*skp, a, pl, sh, wk, cell, row, rank, pl.cluster);
+        if (pbc_item(a, rows, it, cell, row)) p_cell<true>(*skp, a, pl, sh, wk, cell, row, rank, pl.cluster, (int)it);
     }
 }
 
