@@ -87,6 +87,41 @@ def _dftb_flops_per_cell(iters, n=6, nocc=4, npair=3):
     return per_iter * np.asarray(iters, float) + 1000.0 * npair
 
 
+WARM_EVALS = 4   # cells with more SCC iterations than this went through the general path
+
+
+def _warm_products(evals, n, nocc, entries):
+    """FP64 multiply-adds of the matrix products of a warm-started evaluation (n orbitals, o = n_occ, v = n - o):
+    the orthonormal correction S C, C^T S C lower, C E (2 n^3 + n^2 (n + 1) / 2); per evaluation S C_o, the
+    populations, H, H C_o and A_vo (2 n^2 o + n o + n^2 + n o v); the rotation between two of them (2 n o v);
+    A_oo lower (n o (o + 1) / 2), t = A_oo C_o^T (n o^2; a water needs its two hydrogens' rows only) and the
+    given number of entries of P and of W (o each). No eigenproblem is solved."""
+    n, o, ev = (np.asarray(x, float) for x in (n, nocc, evals))
+    v = n - o
+    t = np.where(n > 6, n, 2.0) * o * o
+    return (2 * n ** 3 + n * n * (n + 1) / 2 + ev * (2 * n * n * o + n * o + n * n + n * o * v)
+            + np.maximum(ev - 1, 0) * 2 * n * o * v + n * o * (o + 1) / 2 + t + 2 * o * np.asarray(entries, float))
+
+
+def _warm_flops_per_cell(evals, n=6, nocc=4, npair=3):
+    """FP64 flops of a warm-started cell of waters: its products, P and W between different atoms (n^2 / 2 less
+    9 entries per water), and 1000 per atom pair as in the general count. A water with two evaluations: 2 * 1610
+    + 3000."""
+    n = np.asarray(n, float)
+    return 2 * _warm_products(evals, n, nocc, n * n / 2 - 1.5 * n) + 1000.0 * np.asarray(npair, float)
+
+
+def _periodic_warm_flops_per_cell(evals, n, nocc):
+    """FP64 flops of the products of a warm-started periodic cell (P and W: the lower triangles). The pair sums
+    are not counted, as in the general count."""
+    return 2 * _warm_products(evals, n, nocc, n * (n + 1) / 2)
+
+
+def _flops_by_path(iters, warm, general):
+    """Each cell by the path that its iteration count shows."""
+    return float(sum(warm(i, *c) if i <= WARM_EVALS else general(i, *c) for i, *c in iters))
+
+
 def _periodic_flops_per_cell(iters, n, nocc):
     """FP64 flops of the products one periodic cell needs per time step in the warm-started Gamma-point
     SCC (n orbitals, o = n_occ occupied, v = n - o virtual):
@@ -474,13 +509,17 @@ def _measure_arm(torch, P, w, args, ws, local, precision, charge_model, mlp, flu
         n_orb = 2 * np.diff(sy.cell_offset)          # 6 per water: 2 per atom
         if args.kgrid > 1:   # the same count for each k-point's real form (2n orbitals, 2 n_occ occupied)
             nk = _kgrid_points(args.kgrid)
-            flops = float(sum(nk * _periodic_flops_per_cell(i, 2 * n, 2 * (n * 2 // 3))
-                              for i, n in zip(ev["scc_iters"], n_orb)))
+            n_orb = 2 * n_orb
         else:
-            flops = float(sum(_periodic_flops_per_cell(i, n, n * 2 // 3) for i, n in zip(ev["scc_iters"], n_orb)))
+            nk = 1
+        flops = nk * _flops_by_path(((i, n, n * 2 // 3) for i, n in zip(ev["scc_iters"], n_orb)),
+                                    _periodic_warm_flops_per_cell, _periodic_flops_per_cell)
     else:
-        flops = float(_dftb_flops_per_cell(ev["scc_iters"], *_cell_shapes(sy)).sum())
+        shapes = _cell_shapes(sy)
+        flops = float(np.where(ev["scc_iters"] <= WARM_EVALS, _warm_flops_per_cell(ev["scc_iters"], *shapes),
+                               _dftb_flops_per_cell(ev["scc_iters"], *shapes)).sum())
     generic = not np.all(np.diff(sy.cell_offset) == 3)
+    water_kernel = "k_water_warm" if np.median(ev["scc_iters"]) <= WARM_EVALS else "dftb_kernel<3,6>"
     n_sm = torch.cuda.get_device_properties(local).multi_processor_count
     peak = n_sm * FP64_FLOPS_PER_CLK_SM * SM_MAX_MHZ_NOMINAL * 1e6 / 1e12
     achieved = flops / (dftb_ms * 1e-3) / 1e12
@@ -494,14 +533,19 @@ def _measure_arm(torch, P, w, args, ws, local, precision, charge_model, mlp, flu
     launches = int(phase_cnt.sum()) + (int(phase_cnt[3]) if fd else 0) + \
         2 * (int(phase_cnt[3]) if charge_model == "born_mlp" else 0) + (int(phase_cnt[0]) if mixed else 0) + \
         (int(phase_cnt[0]) if mixed and args.mode_positions == "com" else 0)
+    if args.kgrid > 1 and "clusters of 1 " not in ctx.cavmd_tuning():
+        launches += int(phase_cnt[0])   # the launch over the cells that left the warm path
     arm = {
         "value": value, "unit": "molecule-steps/s", "ms_per_step": max_ms / args.steps,
         "precision": precision, "charge_model": charge_model,
         "config": _config(args.workload, w, charge_model, precision, args.mode_positions, args.kgrid),
         "roofline": {"bound": "alu",
-                     "kernel": "k_dftb_periodic" if periodic else ("k_dftb_generic" if generic else "dftb_kernel<3,6>"),
+                     "kernel": "k_dftb_periodic" if periodic else ("k_dftb_generic" if generic else water_kernel),
                      "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
-                     "traffic": None, "flops_per_launch": flops, "avg_launch_ms": dftb_ms,
+                     "traffic": None, "flops_per_launch": flops,
+                     "flops_note": "FP64 flops of the algorithm by path: the products of the warm-started cells "
+                                   "(no eigenproblem), 11 n^3 and more per iteration of the others; the FP32 start "
+                                   "is not counted", "avg_launch_ms": dftb_ms,
                      "mean_scc_iters": float(np.mean(ev["scc_iters"])),
                      "peak_note": f"FP64 ALU: {n_sm} SMs x 4 FP64 flop/clk x {SM_MAX_MHZ_NOMINAL:.0f} MHz (derived; "
                                   f"no FP64 figure in the measured peaks)",

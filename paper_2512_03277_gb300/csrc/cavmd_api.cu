@@ -467,8 +467,8 @@ int autotune(cavmd_ctx *c) {
     } else {
         c->water_warps = best->a;
         c->water_per_warp = best->b;
-        std::snprintf(buf, sizeof(buf), "dftb_kernel<3,6>: warps_per_block=%d waters_per_warp=%d (%.3f ms); candidates:",
-                      best->a, best->b, best->ms);
+        std::snprintf(buf, sizeof(buf), "dftb_kernel<3,6>%s: warps_per_block=%d waters_per_warp=%d (%.3f ms); candidates:",
+                      c->da.warm_water ? ", warm steps k_water_warm" : "", best->a, best->b, best->ms);
         rep = buf;
         for (auto &cd : cands) {
             std::snprintf(buf, sizeof(buf), " w%d/g%d %.3f ms", cd.a, cd.b, cd.ms);
