@@ -177,15 +177,22 @@ typedef struct {
                                    index (0 = the initial one, then the step number) is a multiple
                                    of this; the paper refreshes every 3 steps. Stale in between.  */
     double fd_step;             /* finite-difference displacement, bohr                      */
-    double scc_tol;             /* max |q_out - q_in| per atom at convergence                */
-    int32_t scc_max_iter;
-    double mixing;              /* linear part of the charge mixing                           */
+    double scc_tol;             /* max |q_out - q_in| per atom at convergence; for warm-started waters
+                                   (atoms in the order of 4, 1 and 1 orbitals) the change of a charge that
+                                   the last residual asks for with the charges' response. Warm-started
+                                   cells take that change into their result.                     */
+    int32_t scc_max_iter;       /* iterations of a cell; a warm-started cell that does not converge in
+                                   min(scc_max_iter, 8) evaluations goes on with as many iterations  */
+    double mixing;              /* linear part of the charge mixing (of cold starts and of cells that
+                                   leave the warm-started path, which does not mix)              */
     int32_t splitting;          /* CAVMD_SPLIT_*                                              */
     int32_t photon_init;        /* CAVMD_PHOTON_*                                             */
     int32_t graph_chunk;        /* steps per captured CUDA graph; 0 = no graph                */
     int32_t device;             /* CUDA device ordinal                                        */
     void *stream;               /* cudaStream_t to run on, or NULL for a library-owned stream */
-    cavmd_alloc_fn dev_alloc;   /* optional device allocator (e.g. a framework's); NULL = cudaMalloc */
+    cavmd_alloc_fn dev_alloc;   /* optional device allocator (e.g. a framework's); NULL = cudaMalloc.
+                                   It returns NULL when it has not the memory (periodic cells then try
+                                   with fewer cells in flight)                                   */
     cavmd_free_fn dev_free;     /* its matching free                                          */
     void *alloc_user;           /* passed back to dev_alloc / dev_free                        */
     int32_t energy_history;     /* steps of energy history kept on the device (>= 1)          */
@@ -197,7 +204,8 @@ typedef struct {
                                    give bitwise identical results); 0: fixed defaults            */
     int32_t scc_history;        /* Anderson mixing history of the cluster kernel: the current and
                                    up to scc_history-1 previous iterates (1..6; 1 = linear mixing).
-                                   Cells of 3 atoms / 6 orbitals use a fixed history of 3.        */
+                                   Cells of 3 atoms / 6 orbitals use a fixed history of 3. Cold starts and
+                                   cells that leave the warm-started path only, as for mixing.    */
     int32_t mode_positions;     /* CAVMD_MODES_FIXED (default) or CAVMD_MODES_CENTRE_OF_MASS    */
     int32_t jacobi_max_sweeps;  /* bound on the Jacobi sweeps of a cold start (the first evaluation,
                                    and the first SCC iteration after cavmd_set_state): 0 = the

@@ -785,7 +785,9 @@ int build_context(cavmd_ctx *c, const cavmd_system *sys, const cavmd_sk_tables *
     std::vector<double> kpts;
     if (sys->lattice && kgrid_points(&c->opt) > 1) kpts = pbc_kpoints(c->opt.kgrid);
     const int nk = (int)(kpts.size() / 4);
-    bool water_order = true;   // every cell: 4, 1 and 1 orbitals in this order, eight electrons
+    // every cell: 4, 1 and 1 orbitals in this order, eight electrons. (k_water_warm fixes the orbital, the atom and
+    // the pair of a lane by its number; a batch with one cell in another order stays with dftb_kernel.)
+    bool water_order = true;
     for (int n = 0; n < N; ++n) {
         int no = 0;
         for (int i = sys->cell_offset[n]; i < sys->cell_offset[n + 1]; ++i) no += sk->norb[sys->species[i]];

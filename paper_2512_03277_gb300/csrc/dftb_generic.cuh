@@ -19,8 +19,8 @@
 //     occupied-virtual generator, C V, and S C_occ for the Mulliken populations;
 //   * four n x n matrices per cell in shared memory: SH (the symmetric S in the strict lower
 //     triangle, the symmetric H0 in the upper triangle and on the diagonal, since S_ii = 1),
-//     C, A and Y, plus the compact generator. A (H2O)_8 cell (48 orbitals) takes about 92 KB, so
-//     two large cells share an SM.
+//     C, A and Y, plus the compact generator and the warm path's n x n_occ buffer. A (H2O)_8 cell (48
+//     orbitals) takes 108 KB, so two large cells share an SM.
 #pragma once
 
 #include "cavmd_internal.cuh"
@@ -276,9 +276,8 @@ struct GWarm {
 // rotation or overlap change, a Hessian or gap that is not safely positive, no convergence): the
 // general path takes it. On success: C (FP64, occupied columns first), q; shift and XB = H C_o of the charges
 // before their last change `moved`.
-// Measured (GB300, one launch of 16,384 clusters (H2O)_1..8, 128 threads per block): 84 -> 24 ms, mean
-// evaluations 2.0 against 10.8 iterations; 301 clusters 4.9 -> 1.1 ms. Bound: the FP64 pipe (65 % busy
-// with 256 threads).
+// Measured (GB300, 16,384 clusters (H2O)_1..8 x 2 steps): 170 -> 48 ms, mean evaluations 2.0 against 10.8
+// iterations; 301 clusters x 4 steps 20.2 -> 3.25 ms. Bound: the FP64 pipe (about 65 % busy).
 template <int T>
 __device__ bool g_warm(const DftbArgs &a, const GWarm &v, double *&C, double *&Y, const double *cw, const Grp<T> &g,
                        int &evals) {

@@ -489,7 +489,7 @@ __device__ __noinline__ void p_settle(const DftbArgs &a, const PbcDev &pl, SH &s
     p_shifts(sh, pl, wk, nat);
 }
 
-// Warm-started cell: the method of k_water_warm and g_warm (dftb_kernel.cu, dftb_generic.cu) for the
+// Warm-started cell: the method of k_water_warm and g_warm (dftb_kernel.cu, dftb_generic.cuh) for the
 // staged products of this kernel and for a set of k-points coupled by the charges.
 //
 // The general path spends about twelve FP64 iterations, Cholesky factors and Jacobi sweeps on iterates
@@ -506,7 +506,7 @@ __device__ __noinline__ void p_settle(const DftbArgs &a, const PbcDev &pl, SH &s
 // columns first (each block its own k-points), sh.q, sh.dq and sh.shift (not for a finite-difference copy), and
 // for the Gamma point Y = H C_o before the last change of the charges and in Mv (FP32) half of that change of A_oo.
 // Measured (GB300, one step): 304 cells of 33 waters 263 -> 76 ms (with the image lists and the Ewald split),
-// 24 cells of 8 waters on 3 x 3 x 3 232 -> 18.8 ms (with clusters of blocks); evaluations 11.8 -> 2.0. Bound: FP64
+// 24 cells of 8 waters on 3 x 3 x 3 232 -> 19.4 ms (with clusters of blocks); evaluations 11.8 -> 2.0. Bound: FP64
 // products (7.5 n^3 multiply-adds a cell) and pair sums, the pipe about 65 % busy.
 template <bool KG, class SH>
 __device__ __noinline__ bool p_warm(const DftbArgs &a, const PbcDev &pl, SH &sh, const PbcMem &wk, const double *Cs,
