@@ -101,3 +101,23 @@ def test_warm_steps_of_wide_k_points(P):
     ctx = P.Context(sy, pa, cs.line_modes(8, 1000.0, 0.001, k_max=0.01), o, lattice=lat)
     ctx.cavmd_step(2)
     assert _check(ctx, sy, _solver(pa, lat, (2, 1, 1))).max() <= 4
+
+
+@pytest.mark.parametrize("grid", [(1, 1, 1), (3, 3, 3)])
+def test_displaced_copies_that_leave_the_warm_path(P, grid):
+    """A displacement of 0.3 bohr changes the overlap by more than the warm path takes: copies go through the
+    general path from their cell's basis. Tolerance: populations to 1e-10 times positions of a few bohr over
+    the displacement, for the two ends of a difference. (At 0.5 bohr two overlaps are not positive definite.)"""
+    sy, lat = _periodic(2, 2)
+    o = P.default_options()
+    o.kgrid[:] = grid
+    o.charge_model = 1       # forward finite differences
+    o.fd_step = 0.3
+    pa = cs.load_water_params()
+    mo = cs.line_modes(8, 1000.0, 0.001, k_max=0.01)
+    ctx = P.Context(sy, pa, mo, o, lattice=lat)
+    b = ctx.cavmd_get_eval()["b"].reshape(-1, 3)
+    for c in range(sy.n_cells):
+        s = slice(sy.cell_offset[c], sy.cell_offset[c + 1])
+        ref = PR.born_fd_periodic(pa, sy.species[s], sy.r[s], lat, np.array(mo.pol), h=0.3, kgrid=grid)
+        assert np.abs(b[s] - ref).max() < 2 * 1e-10 * 20.0 / 0.3
